@@ -69,8 +69,13 @@ typedef enum {
 } eik_status;
 
 /* Tuning knobs.  Zero (or a NULL pointer) selects the default; eik_autotune picks
- * them for a given batch.  Defaults depend on how many independent wavefronts the
- * batch has:
+ * them for a given batch.
+ * A solve whose scheduling options (delta, k_delta, window, band, ctas_per_sm, tile,
+ * arith, sched_flags bits 0-2 and 5) are all zero, without counters, trace or
+ * test_stall, runs the guided kernel, with its own tiles and buckets (one warp per
+ * tile: 8x8 in 2D, 4x4x4 to 8x8x4 in 3D); capacity is then a lower bound.  Otherwise
+ * the defaults below fill in the options that are zero.  They depend on how many
+ * independent wavefronts the batch has:
  *   2D, fewer than 8 sources in the batch: 16x16 tiles, k_delta 16, window 16,
  *     band 16, 1 CTA per SM (latency-bound: one front);
  *   2D, 8 or more sources: 16x8 tiles, k_delta 4, window 16, band 8, 8 CTAs of
@@ -103,7 +108,10 @@ typedef struct {
     double band;           /* in-tile acceptance band in units of (smallest h/v of the tile)
                               / sqrt(ndim), i.e. one cell's travel time; <= 0: default */
     int arith;             /* arithmetic of d-bar: 1 = FP64 unit, 2 = exact emulation on the
-                              integer pipes (same results bit for bit); 0: default */
+                              integer pipes (same results bit for bit); 0: default;
+                              3 = the guided kernel, whatever the other scheduling options
+                              (counters, a trace, test_stall, update 1-3 or sched_flags bits
+                              0-2 and 5 still select the other kernel, as with 0) */
     int sched_flags;       /* bit 0: the look-ahead window follows the lowest bucket holding
                               queued entries only (tiles still running do not hold it);
                               bits 1-2: lane-group d-bar, 0 = automatic (when the batch has

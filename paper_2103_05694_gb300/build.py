@@ -16,9 +16,9 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "_libeik.so")
-SOURCES = ["eik_solver.cu", "eik_api.cu", "eik_selftest.cu", "eik_noalloc.cu", "eik_adjoint.cu",
+SOURCES = ["eik_solver.cu", "eik_guided.cu", "eik_api.cu", "eik_selftest.cu", "eik_noalloc.cu", "eik_adjoint.cu",
            "eik_ablation.cu", "eik_schedules.cu"]
-HEADERS = ["eik_internal.h", "eik_exact.cuh", "eik_forms.cuh", "eik_grid.cuh",
+HEADERS = ["eik_internal.h", "eik_sched.cuh", "eik_exact.cuh", "eik_forms.cuh", "eik_grid.cuh",
            os.path.join("..", "..", "include", "eik.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",

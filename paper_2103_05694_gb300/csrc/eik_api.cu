@@ -55,6 +55,7 @@ constexpr double kKDelta3[2] = {0.75, 0.375};   // single front, many fronts
 constexpr int kSingleFrontCtas3Small = 14;      // 3D tiles of at most 64 cells
 constexpr int kManyFronts = 8;                  // sources at which a solve counts as many fronts
 constexpr int kMaxRetries = 4;
+constexpr int kArithGuided = 3;                 // eik_opts.arith: the guided kernel
 // eik_opts.sched_flags bits of the tomography interface
 constexpr int kFlagSlowness = 1 << 6;     // speed arrays hold slowness s; v = fl(1/s) is used
 constexpr int kFlagSumShared = 1 << 7;    // eik_adjoint: equal outputs receive the ordered sum
@@ -364,15 +365,51 @@ AutoCfg auto_config(int ndim, int64_t total_sources, bool int_arith) {
   return {0, kDefaultKDelta[0], kDefaultBand[0], kDefaultWindow[0]};
 }
 
+int64_t count_cells(const std::vector<HostProblem> &hps) {
+  int64_t n = 0;
+  for (const HostProblem &hp : hps) n += hp.n;
+  return n;
+}
 int64_t count_sources(const std::vector<HostProblem> &hps) {
   int64_t n = 0;
   for (const HostProblem &hp : hps) n += (int64_t)hp.src.size();
   return n;
 }
 
+// Whether a solve runs the guided kernel: a lean solve (no counters, trace, stall
+// test, explicit form or integer arithmetic) whose scheduling options are all
+// automatic.  An option that parametrises the other tile kernel selects it.
+bool use_guided(const eik_opts *o) {
+  if (!o) return true;
+  if (o->counters || o->trace || o->test_stall || o->update || o->schedule) return false;
+  if (o->sched_flags & (1 | 6 | 32)) return false;
+  if (o->arith == kArithGuided) return true;
+  return o->arith == 0 && o->tile == 0 && o->ctas_per_sm <= 0 && o->window <= 0 && !(o->band > 0) &&
+         !(o->delta > 0) && !(o->k_delta > 0);
+}
+// Shape, bucket width, look-ahead and CTAs per SM of a guided solve.  A few
+// fronts are bound by the latency of the visits along them: small tiles.  With
+// many fronts, or one in a large volume, larger tiles cost fewer instructions
+// per cell (88-problem 3D batch: 8x8x4 70 ms, 8x4x4 88 ms, 4x4x4 113 ms; 256^3
+// checkerboard: 8x4x4 12.7 ms, 4x4x4 14.6 ms; one 97 x 131 x 203 grid: 4x4x4
+// 3.7 ms, 8x4x4 4.3 ms; 2D: 8x8 in all cases, 16x8 and 16x16 lost).
+struct GuidedCfg {
+  int shape;        // of the guided shapes
+  double k_delta;
+  int window;
+  int per_sm;       // CTAs (warps) per SM
+};
+GuidedCfg guided_config(int ndim, int64_t total_sources, int64_t cells) {
+  const bool many = total_sources >= kManyFronts;
+  if (ndim == 2) return many ? GuidedCfg{0, 4.0, 16, eik::kGuidedCtas} : GuidedCfg{0, 16.0, 16, 4};
+  const bool large = cells >= (int64_t(1) << 23);
+  if (many) return GuidedCfg{large ? 2 : 0, 0.75, 31, eik::kGuidedCtas};
+  return GuidedCfg{large ? 1 : 0, 0.75, 31, kSingleFrontCtas3Small};
+}
+
 // Tile shape of opts (validated): shape index and cells per axis.  opts.tile 0
 // is automatic; 1..kNumTileShapes name shape tile - 1.
-eik_status tile_shape(const eik_opts *opts, int ndim, int64_t total_sources, int &shape,
+eik_status tile_shape(const eik_opts *opts, int ndim, int64_t total_sources, int64_t cells, int &shape,
                       int64_t &tx, int64_t &ty, int64_t &tz) {
   const int t = opts ? opts->tile : 0;
   const bool int_arith = opts && opts->arith == 2;
@@ -380,7 +417,10 @@ eik_status tile_shape(const eik_opts *opts, int ndim, int64_t total_sources, int
     set_err("opts.tile must be in 0..%d", eik::kNumTileShapes);
     return EIK_EINVAL;
   }
-  shape = t == 0 ? auto_config(ndim, total_sources, int_arith).shape : t - 1;
+  if (use_guided(opts))
+    shape = eik::kGuidedShape0 + guided_config(ndim, total_sources, cells).shape;
+  else
+    shape = t == 0 ? auto_config(ndim, total_sources, int_arith).shape : t - 1;
   if (shape != 0 && int_arith) {
     set_err("integer-pipe arithmetic (arith 2) runs the first tile shape only (opts.tile 0 or 1)");
     return EIK_EINVAL;
@@ -444,7 +484,11 @@ int default_ctas_per_sm(int di, int64_t tile_cells, int64_t total_sources, int w
 // sp already set); else the normal build's count.  Sets sp.lane_group_cells
 // and sp.wide.
 int64_t size_grid(SolveParams &sp, const eik_opts *opts, int ndim, int shape, int64_t tile_cells,
-                  int64_t total_sources, int64_t total_tiles, int sms) {
+                  int64_t cells, int64_t total_sources, int64_t total_tiles, int sms) {
+  if (sp.guided) {
+    const GuidedCfg gc = guided_config(ndim, total_sources, cells);
+    return std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * gc.per_sm, total_tiles));
+  }
   const int occ = eik::persistent_blocks_per_sm(ndim, sp.arith, shape);
   const int occ_wide = eik::persistent_wide_blocks_per_sm(ndim, sp.arith, shape);
   const int per_sm = opts && opts->ctas_per_sm > 0
@@ -610,7 +654,7 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
   }
   int64_t tx, ty, tz;
   int shape = 0;
-  st = tile_shape(opts, ndim, count_sources(hps), shape, tx, ty, tz);
+  st = tile_shape(opts, ndim, count_sources(hps), count_cells(hps), shape, tx, ty, tz);
   if (st != EIK_OK) return st;
   int form = 0;
   st = update_form(opts, ndim, form);
@@ -693,11 +737,14 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
   if (total_tiles >= (int64_t(1) << 32)) { set_err("too many tiles"); return EIK_EINVAL; }
   CK(ws().state.ensure((size_t)total_tiles), "alloc tile state");
   CK(ws().tile_src.ensure((size_t)total_tiles), "alloc tile flags");
-  CK(ws().pend.ensure((size_t)total_tiles * eik::kPendWords), "alloc pending masks");
+  const bool guided = use_guided(opts);   // (the guided kernel defers nothing)
+  if (!guided) CK(ws().pend.ensure((size_t)total_tiles * eik::kPendWords), "alloc pending masks");
 
   // frontier capacity per bucket slot
   uint64_t want_cap = opts && opts->capacity > 0 ? (uint64_t)opts->capacity
                                                  : (uint64_t)total_tiles / 4 + 4096;
+  // a capacity given for the other kernel's tiles and buckets is a lower bound here
+  if (guided) want_cap = std::max<uint64_t>(want_cap, (uint64_t)total_tiles / 4 + 4096);
   want_cap = next_pow2(std::max<uint64_t>(want_cap, opts && opts->capacity > 0 ? 16 : 1024));
   while (want_cap * eik::kNumSlots > kMaxCapEntries && want_cap > 1024) want_cap >>= 1;
   // the ring layout depends on cap; storage only grows.  Entries need no
@@ -721,8 +768,9 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
   CK(cudaMemsetAsync(ws().state.p, 0, (size_t)total_tiles * sizeof(unsigned long long), stream),
      "clear tile states");
   CK(cudaMemsetAsync(ws().tile_src.p, 0, (size_t)total_tiles, stream), "clear tile flags");
-  CK(cudaMemsetAsync(ws().pend.p, 0, (size_t)total_tiles * eik::kPendWords * sizeof(unsigned),
-                     stream), "clear pending masks");
+  if (!guided)
+    CK(cudaMemsetAsync(ws().pend.p, 0, (size_t)total_tiles * eik::kPendWords * sizeof(unsigned),
+                       stream), "clear pending masks");
   CK(cudaMemsetAsync(ws().seq.p, 0, (size_t)(want_cap * eik::kNumSlots) * sizeof(unsigned), stream),
      "clear frontier sequence");
 
@@ -751,6 +799,7 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
   for (auto &P : probs) max_cells = std::max<int64_t>(max_cells, P.nx * P.ny * P.nz);
   CK(eik::launch_init_t_all(ws().probs.p, (int)probs.size(), max_cells, stream), "init_t launch");
 
+  const eik_opts *opts_sched = opts;   // scheduling options that apply
   SolveParams sp;
   std::memset(&sp, 0, sizeof(sp));
   sp.probs = ws().probs.p;
@@ -759,8 +808,15 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
   sp.state = ws().state.p;
   sp.tile_src = ws().tile_src.p;
   sp.pend = ws().pend.p;
-  const AutoCfg ac = auto_config(ndim, total_src, opts && opts->arith == 2);
-  sp.window = (unsigned)(opts && opts->window > 0 ? opts->window : ac.window);
+  AutoCfg ac = auto_config(ndim, total_src, opts && opts->arith == 2);
+  sp.guided = use_guided(opts);
+  if (sp.guided) {
+    const GuidedCfg gc = guided_config(ndim, total_src, count_cells(hps));
+    ac.k_delta = gc.k_delta;
+    ac.window = gc.window;
+    opts_sched = nullptr;
+  }
+  sp.window = (unsigned)(opts_sched && opts_sched->window > 0 ? opts_sched->window : ac.window);
   sp.band = opts && opts->band > 0 ? opts->band : ac.band;
   sp.arith = opts && opts->arith == 2 ? eik::kArithInt : eik::kArithFp64;
   sp.gate_pending_only = opts && (opts->sched_flags & 1) ? 1 : 0;
@@ -779,14 +835,14 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
   sp.timeout_ns = tmo_ms * 1000000ll;
   sp.counters = opts ? opts->counters : 0;
   sp.test_stall = opts ? opts->test_stall : 0;
-  const double k_delta = opts && opts->k_delta > 0 ? opts->k_delta : ac.k_delta;
-  const double delta_fixed = opts && opts->delta > 0 ? opts->delta : 0.0;
+  const double k_delta = opts_sched && opts_sched->k_delta > 0 ? opts_sched->k_delta : ac.k_delta;
+  const double delta_fixed = opts_sched && opts_sched->delta > 0 ? opts_sched->delta : 0.0;
 
   CK(eik::launch_seed(sp, ws().seeds.p, (int64_t)seeds.size(), k_delta, delta_fixed, stream),
      "seed launch");
   int dev_sms = 0;
   CK(cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, ws().device), "SM count");
-  const int64_t grid = size_grid(sp, opts, ndim, shape, tx * ty * tz, total_src, total_tiles, dev_sms);
+  const int64_t grid = size_grid(sp, opts, ndim, shape, tx * ty * tz, count_cells(hps), total_src, total_tiles, dev_sms);
 
   eik_stats acc;
   std::memset(&acc, 0, sizeof(acc));
@@ -1085,6 +1141,12 @@ eik_status eik_autotune(const eik_problem *probs, int nprob, const eik_opts *bas
     if (std::memcmp(&start, &cur, sizeof(cur)) == 0) break;   // no change in a whole pass
   }
   if (st != EIK_OK) { if (ntrials) *ntrials = std::min(n, max_trials); return st; }
+  // the guided kernel against the best of the options above
+  eik_opts guided = cur;
+  guided.arith = kArithGuided;
+  if (use_guided(base) && use_guided(&guided)) {
+    if ((st = consider(guided)) != EIK_OK) { if (ntrials) *ntrials = std::min(n, max_trials); return st; }
+  }
   // frontier capacity from the deepest slot the chosen schedule reaches
   if (!base || base->capacity <= 0) {
     eik_opts o = cur;
@@ -1425,7 +1487,7 @@ eik_status plan_build(eik_plan &pl, std::vector<HostProblem> &hps, const eik_opt
   }
   int64_t tx, ty, tz;
   int shape = 0;
-  eik_status tst = tile_shape(opts, pl.ndim, count_sources(hps), shape, tx, ty, tz);
+  eik_status tst = tile_shape(opts, pl.ndim, count_sources(hps), count_cells(hps), shape, tx, ty, tz);
   if (tst != EIK_OK) return tst;
   int form = 0;
   tst = update_form(opts, pl.ndim, form);
@@ -1526,9 +1588,11 @@ eik_status plan_build(eik_plan &pl, std::vector<HostProblem> &hps, const eik_opt
   if (pl.total_tiles >= (int64_t(1) << 32)) { set_err("too many tiles"); return EIK_EINVAL; }
   CK(pl.state.ensure((size_t)pl.total_tiles), "plan: alloc tile state");
   CK(pl.tile_src.ensure((size_t)pl.total_tiles), "plan: alloc tile flags");
-  CK(pl.pend.ensure((size_t)pl.total_tiles * eik::kPendWords), "plan: alloc pending masks");
+  if (!use_guided(opts))
+    CK(pl.pend.ensure((size_t)pl.total_tiles * eik::kPendWords), "plan: alloc pending masks");
   uint64_t want_cap = opts && opts->capacity > 0 ? (uint64_t)opts->capacity
                                                  : (uint64_t)pl.total_tiles / 2 + 4096;
+  if (use_guided(opts)) want_cap = std::max<uint64_t>(want_cap, (uint64_t)pl.total_tiles / 2 + 4096);
   want_cap = next_pow2(std::max<uint64_t>(want_cap, 16));
   while (want_cap * eik::kNumSlots > kMaxCapEntries && want_cap > 1024) want_cap >>= 1;
   pl.cap = want_cap;
@@ -1552,6 +1616,7 @@ eik_status plan_build(eik_plan &pl, std::vector<HostProblem> &hps, const eik_opt
                      cudaMemcpyHostToDevice, stream), "plan: upload problems");
   CK(cudaStreamSynchronize(stream), "plan: uploads");
 
+  const eik_opts *opts_sched = opts;   // scheduling options that apply
   SolveParams &sp = pl.sp;
   std::memset(&sp, 0, sizeof(sp));
   sp.probs = pl.probs_d.p;
@@ -1568,8 +1633,15 @@ eik_status plan_build(eik_plan &pl, std::vector<HostProblem> &hps, const eik_opt
   sp.timeout_ns = tmo_ms * 1000000ll;
   sp.counters = opts ? opts->counters : 0;
   sp.test_stall = 0;
-  const AutoCfg ac = auto_config(pl.ndim, count_sources(hps), opts && opts->arith == 2);
-  sp.window = (unsigned)(opts && opts->window > 0 ? opts->window : ac.window);
+  AutoCfg ac = auto_config(pl.ndim, count_sources(hps), opts && opts->arith == 2);
+  sp.guided = use_guided(opts);
+  if (sp.guided) {
+    const GuidedCfg gc = guided_config(pl.ndim, count_sources(hps), count_cells(hps));
+    ac.k_delta = gc.k_delta;
+    ac.window = gc.window;
+    opts_sched = nullptr;
+  }
+  sp.window = (unsigned)(opts_sched && opts_sched->window > 0 ? opts_sched->window : ac.window);
   sp.band = opts && opts->band > 0 ? opts->band : ac.band;
   sp.arith = opts && opts->arith == 2 ? eik::kArithInt : eik::kArithFp64;
   sp.gate_pending_only = opts && (opts->sched_flags & 1) ? 1 : 0;
@@ -1579,12 +1651,12 @@ eik_status plan_build(eik_plan &pl, std::vector<HostProblem> &hps, const eik_opt
   sp.visit_budget = sp.track_changes ? (unsigned long long)pl.total_tiles * 256ull + 4096ull : 0ull;
   sp.trace = nullptr;
   sp.trace_cap = 0;
-  pl.k_delta = opts && opts->k_delta > 0 ? opts->k_delta : ac.k_delta;
-  pl.delta_fixed = opts && opts->delta > 0 ? opts->delta : 0.0;
+  pl.k_delta = opts_sched && opts_sched->k_delta > 0 ? opts_sched->k_delta : ac.k_delta;
+  pl.delta_fixed = opts_sched && opts_sched->delta > 0 ? opts_sched->delta : 0.0;
   pl.from_slowness = from_slowness(opts);
   int sms = 0;
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, pl.device), "SM count");
-  pl.grid = (int)size_grid(sp, opts, pl.ndim, shape, tx * ty * tz, pl.nseeds, pl.total_tiles, sms);
+  pl.grid = (int)size_grid(sp, opts, pl.ndim, shape, tx * ty * tz, count_cells(hps), pl.nseeds, pl.total_tiles, sms);
   return EIK_OK;
 }
 
@@ -1622,8 +1694,9 @@ eik_status eik_plan_enqueue(eik_plan *pl, void *stream) {
   CK(cudaMemsetAsync(pl->state.p, 0, (size_t)pl->total_tiles * sizeof(unsigned long long), s),
      "clear tile states");
   CK(cudaMemsetAsync(pl->tile_src.p, 0, (size_t)pl->total_tiles, s), "clear tile flags");
-  CK(cudaMemsetAsync(pl->pend.p, 0, (size_t)pl->total_tiles * eik::kPendWords * sizeof(unsigned), s),
-     "clear pending masks");
+  if (!pl->sp.guided)
+    CK(cudaMemsetAsync(pl->pend.p, 0, (size_t)pl->total_tiles * eik::kPendWords * sizeof(unsigned), s),
+       "clear pending masks");
   CK(cudaMemsetAsync(pl->seq.p, 0, (size_t)(pl->cap * eik::kNumSlots) * sizeof(unsigned), s),
      "clear frontier sequence");
   for (size_t j = 0; j < pl->speeds.size(); ++j) {

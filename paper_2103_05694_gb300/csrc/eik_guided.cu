@@ -1,0 +1,534 @@
+// Guided tile kernel: the default of lean solves with automatic options.
+//
+// The asynchronous tile schedule of eik_solver.cu (same buckets, claims and
+// activations) with another way to relax a claimed tile.  That kernel finds
+// the order of a tile's cells by exact arithmetic: every round of provisional
+// d-bar values costs two block barriers and a dependent chain, and a cell is
+// evaluated 6 (3D batch) to 33 times (2D section).  Here one warp owns a tile
+// and a visit has two parts:
+//
+//  1. Order.  The tile's values and halo become float offsets g from their
+//     minimum, and the first-order update is relaxed in FP32 until nothing falls
+//     by more than a thousandth of a cell's r (a row of 32 cells takes about 80
+//     warp instructions).
+//  2. Exact.  Each cell that may change is evaluated by d-bar once, after its
+//     neighbours in the tile with smaller g.  The order is kept as bit sets over
+//     the tile (one 32-bit word per lane): a cell is ready when none of the
+//     neighbours it waits for is left in the set of cells to do, a handful of
+//     shifts and masks per round for the whole tile, and the ready cells are
+//     packed onto the lanes.
+//  Then every cell is checked against the neighbours it did not wait for: one
+//  that fell below it since makes it be evaluated again, until there are none.
+//
+// g only orders the evaluations.  When the visit ends, no neighbour has fallen
+// below a cell since the cell's last evaluation, so the fixed point and its
+// bits are those of any schedule (Theorem 1), whatever the floats say.  Nothing
+// is deferred inside a visit: the look-ahead window only limits which tiles are
+// taken.
+//
+// What bounds it: with many fronts, instructions (88-problem 3D batch: issue 52 %
+// at 4.75 warps per scheduler, the instruction cache close to its request rate,
+// so loops are rolled and the scheduler's functions are not inlined: 218 -> 75 ms
+// while this was written); with one front, the latency of the visits along it
+// (about 1300 cycles per round of exact evaluations).  Evaluations per cell: 2.5
+// (batch) and 4 (checkerboard) against 6.1 and 11.2 in the other kernel.
+// Measured against that kernel with the same d-bar (us): 129^2 grid 796 -> 613,
+// layered section 12286 -> 9417, 256^3 checkerboard 17345 -> 12597, 88-problem
+// batch 115674 -> 61437.
+// Tried and dropped: a visit limit inside the tile (narrow windows leave partial
+// tiles: batch 75 -> 139 ms at a quarter of the bucket width); waiting while a
+// neighbour tile is being visited (visits halve, the wait costs more); skipping
+// cells no neighbour has fallen below (batch 71.7 -> 74.1 ms); more warps per SM
+// with fewer registers (69.0 -> 73.5 ms at 23).
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "eik_exact.cuh"
+#include "eik_internal.h"
+#define EIK_SCHED_FN __device__ __noinline__   // one copy each: the kernel is bound by instruction fetch
+#include "eik_sched.cuh"
+
+namespace eik {
+namespace {
+
+constexpr float kSettled = 1e-3f;   // falls below this many r stop the FP32 relaxation
+constexpr float kInfF = __builtin_huge_valf();
+
+// A non-negative double (bit pattern) times 2^-se as a float, truncated; +inf stays.
+__device__ __forceinline__ float to_f_scaled(unsigned long long u, int se) {
+  const int e = static_cast<int>(u >> 52) - 1023 + 127 - se;
+  if (u == 0ull || e <= 0) return 0.0f;
+  if (e >= 255) return kInfF;
+  return __int_as_float((e << 23) | static_cast<int>((u >> 29) & 0x7fffffu));
+}
+
+// (v - base) times 2^-se as a float for bit patterns v >= base >= 0, without the
+// FP64 pipe: the significands' integer difference where v lies within 8
+// binades of base, else the difference of the floats.
+__device__ __forceinline__ float offset_f(unsigned long long v, unsigned long long base, int se) {
+  constexpr unsigned long long kFrac = (1ull << 52) - 1, kHid = 1ull << 52;
+  const int eb = static_cast<int>(base >> 52), d = static_cast<int>(v >> 52) - eb;
+  if (eb == 0 || d > 8) return to_f_scaled(v, se) - (v < kInfBits ? to_f_scaled(base, se) : 0.0f);
+  const unsigned long long x = (((v & kFrac) | kHid) << d) - ((base & kFrac) | kHid);
+  const float f = fmaf(__uint2float_rn(static_cast<unsigned>(x >> 32)), 4294967296.0f,
+                       __uint2float_rn(static_cast<unsigned>(x)));
+  const int e = eb - 1075 - se;                   // unit 2^(eb - 1075)
+  const int e1 = e < -126 ? -126 : e > 126 ? 126 : e, e2 = e - e1 < -126 ? -126 : e - e1;
+  return f * __int_as_float((127 + e1) << 23) * __int_as_float((127 + (e2 > 0 ? 126 : e2)) << 23);
+}
+
+// First-order update in FP32 from the axis minima (offsets; +inf allowed), r = h / v.
+template <int D>
+__device__ __forceinline__ float root_f(const float (&a)[D], float r) {
+  float lo = fminf(a[0], a[1]), hi = fmaxf(a[0], a[1]), top = 0.0f;
+  if (D == 3) {
+    top = fmaxf(hi, a[D - 1]);
+    const float m = fminf(hi, a[D - 1]);
+    hi = fmaxf(lo, m);
+    lo = fminf(lo, m);
+  }
+  float u = r;
+  const float b1 = hi - lo;               // NaN when both are +inf: one-sided
+  if (b1 < r) {
+    const float rr = r * r;
+    u = 0.5f * (b1 + ffa::sqrt_est(fmaf(-b1, b1, 2.0f * rr)));
+    if (D == 3) {
+      const float b2 = top - lo;
+      if (b2 < u) {
+        const float s = b1 + b2, q = fmaf(b1, b1, b2 * b2);
+        const float disc = fmaxf(fmaf(s, s, -3.0f * (q - rr)), 1e-30f);
+        u = (s + ffa::sqrt_est(disc)) * (1.0f / 3.0f);
+      }
+    }
+  }
+  return lo + u;
+}
+
+// Bit sets over a tile's cells: lane k < NC holds the word of cells 32 k .. 32 k + 31
+// (the other lanes 0).  For every cell q the bit of cell q + d; bits whose
+// neighbour is off the tile mean nothing and are masked by the caller.
+template <int d>
+__device__ __forceinline__ unsigned nbr_bits(unsigned w, bool across) {
+  constexpr int m = d < 0 ? -d : d;
+  if (m >= 32) {
+    if (d > 0) return __shfl_down_sync(kFull, w, m / 32);
+    const unsigned v = __shfl_up_sync(kFull, w, m / 32);
+    return (threadIdx.x & 31) >= m / 32 ? v : 0u;
+  }
+  unsigned r = d > 0 ? w >> m : w << m;
+  if (across) {        // the neighbour may be in the next word
+    if (d > 0) {
+      r |= __shfl_down_sync(kFull, w, 1) << (32 - m);
+    } else {
+      const unsigned v = __shfl_up_sync(kFull, w, 1) >> (32 - m);
+      r |= (threadIdx.x & 31) > 0 ? v : 0u;
+    }
+  }
+  return r;
+}
+
+template <int D, int TX, int TY, int TZ>
+struct GTile {
+  static constexpr int NT = TX * TY * TZ, NC = NT / 32;
+  static constexpr int HZ = D == 3 ? 1 : 0;
+  static constexpr int SX = TX + 2, SY = TY + 2, SZ = TZ + 2 * HZ, NS = SX * SY * SZ;
+  double t[NS];                    // exact values with halo
+  unsigned long long c[NT];
+  float g[NS];                     // predicted offsets with halo
+  float r[NT];                     // h / v
+  unsigned char list[NT];
+  unsigned char fell[NT];          // 1: fell since the last look
+};
+
+template <int D, int TX, int TY, int TZ>
+__global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) {
+  using S = GTile<D, TX, TY, TZ>;
+  constexpr int NT = S::NT, NC = S::NC, HZ = S::HZ, SX = S::SX, SY = S::SY;
+  static_assert(NT % 32 == 0 && NT <= 256, "whole warps, 8-bit list entries");
+  constexpr int kStride[3] = {1, SX, SX * SY};
+  constexpr int kTile[3] = {TX, TY, TZ};
+  __shared__ S s;
+  const int lane = threadIdx.x;
+  const float inv_delta = static_cast<float>(p.ctl->inv_delta);
+  const int se = p.ctl->scale_exp;
+  const unsigned lt_mask = (1u << lane) - 1u;
+  long long idle_since = 0;
+  auto pos_of = [](int q) { return ((q / (TX * TY) + HZ) * SY + (q / TX) % TY + 1) * SX + q % TX + 1; };
+  // the bits of the neighbours across face j (-x, +x, -y, +y, -z, +z)
+  auto nbrs = [](unsigned w, int j) -> unsigned {
+    switch (j) {
+      case 0: return nbr_bits<-1>(w, false);
+      case 1: return nbr_bits<1>(w, false);
+      case 2: return nbr_bits<-TX>(w, TX * TY > 32);
+      case 3: return nbr_bits<TX>(w, TX * TY > 32);
+      case 4: return nbr_bits<-TX * TY>(w, true);
+      default: return nbr_bits<TX * TY>(w, true);
+    }
+  };
+
+#pragma unroll 1
+  for (;;) {
+    long long tile = -1;
+    int faces = 0;
+    unsigned slot = 0, lo = 0;
+#pragma unroll 1
+    for (;;) {
+      const unsigned long long e = pop_entry(p, idle_since, slot, lo);
+      if (e == kEmpty) break;
+      const unsigned long long tl = e & 0xffffffffull;
+      int f = -1;
+      if (lane == 0) f = try_claim(p, tl, static_cast<unsigned>(e >> 32));
+      f = __shfl_sync(kFull, f, 0);
+      if (f >= 0) { tile = static_cast<long long>(tl); faces = f; break; }
+      if (lane == 0) {
+        atomicAdd(&p.ctl->run[slot * kCounterPad], 0xffffffffu);
+        atomicAdd(&p.ctl->work, -1);
+      }
+    }
+    if (tile < 0) break;
+    idle_since = 0;
+    __threadfence();      // the claim is ordered before the tile's loads
+    const Prob &P = p.probs[find_prob(p, static_cast<unsigned long long>(tile))];
+    int64_t x0, y0, z0;
+    {   // fewer than 2^32 tiles: 32-bit divisions
+      const unsigned lt = static_cast<unsigned>(tile - P.tile_base), ntx = static_cast<unsigned>(P.ntx),
+                     nty = static_cast<unsigned>(P.nty);
+      const unsigned rest = lt / ntx, tz = rest / nty;
+      x0 = static_cast<int64_t>(lt - rest * ntx) * TX;
+      y0 = static_cast<int64_t>(rest - tz * nty) * TY;
+      z0 = static_cast<int64_t>(tz) * TZ;
+    }
+    const int64_t sy = P.nx, sz = P.nx * P.ny, first = z0 * sz + y0 * sy + x0;
+    double *const T0 = P.t + first;      // the tile's first cell
+    // the grid in tile coordinates, as far as the tile and its halo reach
+    const int xlo = x0 > 0 ? -1 : 0, ylo = y0 > 0 ? -1 : 0, zlo = z0 > 0 ? -1 : 0;
+    const int xhi = P.nx - x0 > TX ? TX + 1 : static_cast<int>(P.nx - x0);
+    const int yhi = P.ny - y0 > TY ? TY + 1 : static_cast<int>(P.ny - y0);
+    const int zhi = P.nz - z0 > TZ ? TZ + 1 : static_cast<int>(P.nz - z0);
+    unsigned fixed_w = 0u;               // sources and cells off the grid: word k in lane k
+    const bool has_src = p.tile_src[tile] != 0;
+#pragma unroll 4
+    for (int k = 0; k < NC; ++k) {
+      const int q = k * 32 + lane;
+      const int ix = q % TX, iy = (q / TX) % TY, iz = q / (TX * TY);
+      const bool in = ix < xhi && iy < yhi && iz < zhi;
+      const int64_t off = iz * sz + iy * sy + ix;
+      const double tv = in ? ld_time(T0 + off) : from_bits(kInfBits);
+      const unsigned long long cv =
+          in ? static_cast<unsigned long long>(__ldg(reinterpret_cast<const long long *>(P.c) + first + off)) : 0ull;
+      s.t[pos_of(q)] = tv;
+      s.c[q] = cv;
+      s.fell[q] = 0;
+      const float cf = to_f_scaled(cv, 2 * se);
+      s.r[q] = cf > 0.0f ? ffa::sqrt_est(cf) : 0.0f;
+      const unsigned b = __ballot_sync(kFull, !in);
+      if (lane == k) fixed_w = b;
+    }
+    if (has_src) {
+#pragma unroll 1
+      for (int k = 0; k < NC; ++k) {
+        const int q = k * 32 + lane;
+        const unsigned b = __ballot_sync(kFull, is_source(P, first + (q / (TX * TY)) * sz + ((q / TX) % TY) * sy + q % TX));
+        if (lane == k) fixed_w |= b;
+      }
+    }
+
+    // A claimed tile is worked on until no neighbour has re-activated it meanwhile.
+#pragma unroll 1
+    for (;;) {
+      {  // halo faces: y (x fastest: coalesced), z, x
+        constexpr int FX = TY * TZ, FY = TX * TZ, FZ = (D == 3) ? TX * TY : 0;
+        constexpr int H = 2 * FX + 2 * FY + 2 * FZ;
+#pragma unroll 4
+        for (int i = lane; i < H; i += 32) {
+          int ix, iy, iz;                // tile coordinates, -1 .. extent
+          if (i < 2 * FY) {
+            const int j = i % FY;
+            ix = j % TX; iz = j / TX; iy = i < FY ? -1 : TY;
+          } else if (i < 2 * FY + 2 * FZ) {
+            const int k = i - 2 * FY, j = k % (FZ > 0 ? FZ : 1);
+            ix = j % TX; iy = j / TX; iz = k < FZ ? -1 : TZ;
+          } else {
+            const int k = i - 2 * FY - 2 * FZ, j = k % FX;
+            iy = j % TY; iz = j / TY; ix = k < FX ? -1 : TX;
+          }
+          const bool in = ix >= xlo && ix < xhi && iy >= ylo && iy < yhi && iz >= zlo && iz < zhi;
+          s.t[((iz + HZ) * SY + iy + 1) * SX + ix + 1] =
+              in ? ld_time(T0 + iz * sz + iy * sy + ix) : from_bits(kInfBits);
+        }
+      }
+      __syncwarp();
+
+      // cells to evaluate: every cell (a seeded tile), or those next to a changed
+      // halo value that is below theirs
+      unsigned need_w = (faces & (1 << kFaceFull)) ? kFull : 0u;
+      unsigned long long base = kInfBits;
+#pragma unroll 1
+      for (int k = 0; k < NC; ++k) {
+        const int q = k * 32 + lane, ps = pos_of(q);
+        const int cc[3] = {q % TX, (q / TX) % TY, q / (TX * TY)};
+        const unsigned long long tb = bits_of(s.t[ps]);
+        bool want = false;
+        base = umin64(base, tb);
+#pragma unroll
+        for (int j = 0; j < 2 * D; ++j) {
+          const int ax = j >> 1;
+          if (cc[ax] != ((j & 1) ? kTile[ax] - 1 : 0)) continue;
+          const unsigned long long hv = bits_of(s.t[ps + ((j & 1) ? kStride[ax] : -kStride[ax])]);
+          base = umin64(base, hv);
+          want = want || (((faces >> j) & 1) && hv < tb);
+        }
+        const unsigned b = __ballot_sync(kFull, want);
+        if (lane == k) need_w |= b;
+      }
+      need_w = lane < NC ? need_w & ~fixed_w : 0u;
+      unsigned changed_w = 0u;
+      if (__any_sync(kFull, need_w != 0u)) {
+        base = warp_min64(base);
+        // offsets from the smallest value, in units of 2^se
+#pragma unroll 1
+        for (int i = lane; i < S::NS; i += 32) s.g[i] = offset_f(bits_of(s.t[i]), base, se);
+        unsigned fixed = 0u;                    // bit k: this lane's cell k
+#pragma unroll
+        for (int k = 0; k < NC; ++k) fixed |= ((__shfl_sync(kFull, fixed_w, k) >> lane) & 1u) << k;
+        __syncwarp();
+        // 1. order: relax in FP32 by rows of 32 cells, up and down by turns, each row
+        // while one of its neighbour rows (or itself) has fallen since its last turn
+        unsigned stale = (1u << NC) - 1u;
+        constexpr int kReach = (TX * TY > 32 ? TX * TY : 32) / 32;   // rows hold neighbours up to +-kReach
+#pragma unroll 1
+        for (int it = 0; stale && it < 4 * NT; ++it) {
+#pragma unroll 1
+          for (int kk = 0; kk < NC; ++kk) {
+            const int k = (it & 1) ? NC - 1 - kk : kk;
+            if (!((stale >> k) & 1u)) continue;
+            const int q = k * 32 + lane, ps = pos_of(q);
+            float a[D];
+#pragma unroll
+            for (int ax = 0; ax < D; ++ax) a[ax] = fminf(s.g[ps - kStride[ax]], s.g[ps + kStride[ax]]);
+            const float r = s.r[q];
+            const float nv = root_f<D>(a, r);
+            const bool fell = !((fixed >> k) & 1u) && nv < s.g[ps] - kSettled * r;
+            if (fell) s.g[ps] = nv;
+            stale &= ~(1u << k);
+            if (__any_sync(kFull, fell)) {
+              // rows k, k +- 1, and in 3D tiles of two rows per slice k +- 2
+              unsigned near = (7u << k) >> 1;
+              if (D == 3 && kReach == 2) near |= (17u << k) >> 2;
+              stale |= near & ((1u << NC) - 1u);
+            }
+            __syncwarp();
+          }
+        }
+        // a cell that will be evaluated can change only cells of larger g
+        float g_need = kInfF;
+#pragma unroll 1
+        for (int k = 0; k < NC; ++k)
+          if ((__shfl_sync(kFull, need_w, k) >> lane) & 1u) g_need = fminf(g_need, s.g[pos_of(k * 32 + lane)]);
+        g_need = __uint_as_float(__reduce_min_sync(kFull, __float_as_uint(g_need)));
+        unsigned todo_w = 0u;                   // cells to evaluate
+        unsigned up_w[2 * D];                   // cells that wait for their neighbour across face j
+#pragma unroll
+        for (int j = 0; j < 2 * D; ++j) up_w[j] = 0u;
+#pragma unroll 1
+        for (int k = 0; k < NC; ++k) {
+          const int q = k * 32 + lane, ps = pos_of(q);
+          const int cc[3] = {q % TX, (q / TX) % TY, q / (TX * TY)};
+          const float gq = s.g[ps];
+          const unsigned be = __ballot_sync(kFull, gq >= g_need && gq < kInfF);
+          if (lane == k) todo_w = be;
+#pragma unroll
+          for (int j = 0; j < 2 * D; ++j) {
+            const int ax = j >> 1;
+            const unsigned b = __ballot_sync(kFull, cc[ax] != ((j & 1) ? kTile[ax] - 1 : 0) &&
+                                                        s.g[ps + ((j & 1) ? kStride[ax] : -kStride[ax])] < gq);
+            if (lane == k) up_w[j] = b;
+          }
+        }
+        todo_w = (todo_w | need_w) & ~fixed_w;
+#pragma unroll
+        for (int j = 0; j < 2 * D; ++j) up_w[j] &= nbrs(todo_w, j) & todo_w;
+        // 2. exact evaluations in that order
+        bool ordered = true;
+#pragma unroll 1
+        for (unsigned round = 0;; ++round) {
+          if (round >= kMaxRounds) {
+            if (lane == 0) raise_status(p.ctl, kEtimeout, 7);
+            break;
+          }
+          unsigned ready_w = todo_w;
+          if (ordered) {
+#pragma unroll
+            for (int j = 0; j < 2 * D; ++j) ready_w &= ~(up_w[j] & nbrs(todo_w, j));
+          }
+          // the set's cells as a list: every lane picks its bit of each word (few
+          // words: the shorter chain), or each word's lane writes its bits (many:
+          // fewer instructions)
+          int n = 0;
+          if constexpr (NC <= 2) {
+#pragma unroll
+            for (int k = 0; k < NC; ++k) {
+              const unsigned w = __shfl_sync(kFull, ready_w, k);
+              if ((w >> lane) & 1u) s.list[n + __popc(w & lt_mask)] = static_cast<unsigned char>(k * 32 + lane);
+              n += __popc(w);
+            }
+          } else {
+            const int own = __popc(ready_w);
+            n = own;
+#pragma unroll
+            for (int o = 1; o < NC; o <<= 1) {
+              const int v = __shfl_up_sync(kFull, n, o);
+              if (lane >= o) n += v;
+            }
+            int at = n - own;
+            n = __shfl_sync(kFull, n, NC - 1);
+#pragma unroll 1
+            for (unsigned w = ready_w; w; w &= w - 1u)
+              s.list[at++] = static_cast<unsigned char>(lane * 32 + __ffs(w) - 1);
+          }
+          __syncwarp();
+          if (n > 0) {
+            todo_w &= ~ready_w;
+#pragma unroll 1
+            for (int b = lane; b < ((n + 31) & ~31); b += 32) {
+              if (b < n) {
+                const int q = s.list[b], ps = pos_of(q);
+                unsigned long long a[D];
+                const unsigned long long best = bits_of(s.t[ps]);
+#pragma unroll
+                for (int ax = 0; ax < D; ++ax)
+                  a[ax] = umin64(bits_of(s.t[ps - kStride[ax]]), bits_of(s.t[ps + kStride[ax]]));
+                unsigned long long nv;
+                if (hw::relax<D>(best, a, s.c[q], nv)) {
+                  s.t[ps] = from_bits(nv);
+                  s.fell[q] = 1;
+                }
+              }
+            }
+            __syncwarp();
+            if (ordered) continue;
+          }
+          // All listed cells are evaluated.  A cell is right unless a neighbour it
+          // did not wait for has fallen below it since: list those, in any order.
+          unsigned now_w = 0u, redo_w = 0u, below_w[2 * D];
+#pragma unroll
+          for (int j = 0; j < 2 * D; ++j) below_w[j] = 0u;
+#pragma unroll 1
+          for (int k = 0; k < NC; ++k) {
+            const int q = k * 32 + lane, ps = pos_of(q);
+            const int cc[3] = {q % TX, (q / TX) % TY, q / (TX * TY)};
+            const unsigned b = __ballot_sync(kFull, s.fell[q] != 0);
+            s.fell[q] = 0;
+            if (lane == k) now_w = b;
+            const unsigned long long tb = bits_of(s.t[ps]);
+#pragma unroll
+            for (int j = 0; j < 2 * D; ++j) {
+              const int ax = j >> 1;
+              const unsigned bj = __ballot_sync(
+                  kFull, cc[ax] != ((j & 1) ? kTile[ax] - 1 : 0) &&
+                             bits_of(s.t[ps + ((j & 1) ? kStride[ax] : -kStride[ax])]) < tb);
+              if (lane == k) below_w[j] = bj;
+            }
+          }
+          changed_w |= now_w;
+          if (!__any_sync(kFull, now_w != 0u)) break;
+#pragma unroll
+          for (int j = 0; j < 2 * D; ++j)
+            redo_w |= below_w[j] & nbrs(now_w, j) & ~(ordered ? up_w[j] : 0u);
+          todo_w = redo_w & ~fixed_w;
+          ordered = false;
+          if (!__any_sync(kFull, todo_w != 0u)) break;
+        }
+      }
+
+      // commit, and the smallest committed time per face that is below the
+      // halo value across it (only such a value can change the cell there)
+      if (__any_sync(kFull, changed_w != 0u)) {
+        unsigned fm_any = 0u;
+        unsigned long long fm[2 * D];
+#pragma unroll
+        for (int j = 0; j < 2 * D; ++j) fm[j] = kInfBits;
+#pragma unroll 1
+        for (int k = 0; k < NC; ++k) {
+          if (!((__shfl_sync(kFull, changed_w, k) >> lane) & 1u)) continue;
+          const int q = k * 32 + lane, ps = pos_of(q);
+          const int cc[3] = {q % TX, (q / TX) % TY, q / (TX * TY)};
+          const unsigned long long tb = bits_of(s.t[ps]);
+          // only this tile's visit writes its cells: a plain store
+          st_rlx(reinterpret_cast<unsigned long long *>(T0 + cc[2] * sz + cc[1] * sy + cc[0]), tb);
+#pragma unroll
+          for (int j = 0; j < 2 * D; ++j) {
+            const int ax = j >> 1;
+            if (cc[ax] != ((j & 1) ? kTile[ax] - 1 : 0)) continue;
+            if (tb < bits_of(s.t[ps + ((j & 1) ? kStride[ax] : -kStride[ax])])) fm[j] = umin64(fm[j], tb);
+          }
+        }
+        unsigned long long mine = kInfBits;
+#pragma unroll
+        for (int j = 0; j < 2 * D; ++j) {
+          if (!__any_sync(kFull, fm[j] < kInfBits)) continue;
+          const unsigned long long v = warp_min64(fm[j]);
+          if (lane == j) mine = v;
+          fm_any |= 1u << j;
+        }
+        __threadfence();
+        __syncwarp();
+        if ((fm_any >> lane) & 1u) {
+          const int ax = lane >> 1, up = lane & 1;
+          const int64_t tc[3] = {x0 / TX, y0 / TY, z0 / TZ};
+          const int64_t ext = ax == 0 ? P.ntx : ax == 1 ? P.nty : P.ntz;
+          const int64_t moved = (ax == 0 ? tc[0] : ax == 1 ? tc[1] : tc[2]) + (up ? 1 : -1);
+          if (moved >= 0 && moved < ext) {
+            const int64_t step = ax == 0 ? 1 : ax == 1 ? P.ntx : P.ntx * P.nty;
+            activate(p, static_cast<unsigned long long>(tile + (up ? step : -step)), 1u << (lane ^ 1),
+                     bucket_of_time(mine, inv_delta));
+          }
+        }
+        __syncwarp();
+        __threadfence();
+      }
+      // continue on this tile with its new faces if it was re-activated meanwhile
+      int cont = 0;
+      if (lane == 0) {
+        unsigned long long old = ld_rlx(&p.state[tile]);
+        if (state_of(old) == kStDirty) {
+          const unsigned long long prev = atomicCAS(&p.state[tile], old, make_state(kStRunning, 0, 0));
+          if (prev == old) {
+            cont = 0x100 | static_cast<int>(faces_of(old));
+            __threadfence();   // the claim of the new work before the halo loads
+          }
+        }
+      }
+      cont = __shfl_sync(kFull, cont, 0);
+      if (!cont) break;
+      faces = cont & 0x7f;
+    }
+    if (lane == 0) {
+      finish_tile(p, static_cast<unsigned long long>(tile));
+      __threadfence();
+      atomicAdd(&p.ctl->run[slot * kCounterPad], 0xffffffffu);
+      atomicAdd(&p.ctl->work, -1);
+    }
+    __syncwarp();
+  }
+}
+
+template <int D, int TX, int TY, int TZ>
+cudaError_t run_guided(const SolveParams &p, int grid, cudaStream_t stream) {
+  guided_kernel<D, TX, TY, TZ><<<grid, 32, 0, stream>>>(p);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_guided(const SolveParams &p, int grid, cudaStream_t stream) {
+  note_launches(1);
+  if (p.ndim == 2) return run_guided<2, 8, 8, 1>(p, grid, stream);
+  switch (p.tile_shape - kGuidedShape0) {
+    case 0: return run_guided<3, 4, 4, 4>(p, grid, stream);
+    case 1: return run_guided<3, 8, 4, 4>(p, grid, stream);
+    default: return run_guided<3, 8, 8, 4>(p, grid, stream);
+  }
+}
+
+}  // namespace eik

@@ -54,7 +54,8 @@ struct Ctl {
   double delta;             // bucket width used
   double inv_delta;
   unsigned long long rmin_bits;   // smallest r (bit pattern; all r > 0)
-  int pad3[22];
+  int scale_exp;            // binary exponent of the mean r (the guided kernel's float unit)
+  int pad3[21];
   unsigned long long stats[kNumStats];
   unsigned long long error_info[4];   // where a wait gave up / what was invalid
   unsigned long long trace_n;         // trace records written (may exceed the capacity)
@@ -112,6 +113,7 @@ struct SolveParams {
   unsigned long long trace_cap;
   int wide;                       // lean launches of 4x4x4 3D tiles: the build compiled for
                                   // EIK_WIDE_CTAS_64 CTAs per SM (fewer registers)
+  int guided;                     // 1: the guided kernel (eik_guided.cu; lean solves only)
 };
 
 // One tile visit, for timeline analysis (opts.trace).
@@ -151,7 +153,16 @@ constexpr int resident_ctas(int tile_cells) {
 struct TileShape {
   int tx, ty, tz;
 };
+// The guided kernel's own shapes (one warp per tile) and the CTAs of one warp
+// per SM that its registers are bounded for.
+constexpr int kGuidedShape0 = kNumTileShapes;
+constexpr int kGuidedCtas = 20;
 __host__ __device__ inline TileShape tile_shape_of(int ndim, int shape) {
+  if (shape >= kGuidedShape0) {
+    const int g = shape - kGuidedShape0;
+    if (ndim == 3) return g == 0 ? TileShape{4, 4, 4} : g == 1 ? TileShape{8, 4, 4} : TileShape{8, 8, 4};
+    return TileShape{8, 8, 1};
+  }
   if (ndim == 3) {
     switch (shape) {
       case 1: return TileShape{16, 4, 4};
@@ -207,6 +218,8 @@ cudaError_t launch_seed(const SolveParams &p, const SeedItem *items, int64_t nit
 cudaError_t launch_reseed(const SolveParams &p, const Prob *host_probs, int nprob,
                           cudaStream_t stream);
 cudaError_t launch_persistent(const SolveParams &p, int grid, cudaStream_t stream);
+// The guided kernel on its own tile shapes (tile_shape >= kGuidedShape0).
+cudaError_t launch_guided(const SolveParams &p, int grid, cudaStream_t stream);
 cudaError_t launch_count_finite(const Prob *host_probs, int nprob, unsigned long long *out,
                                 cudaStream_t stream);
 // Finite times over every problem of a batch in one launch (adds into *out).
