@@ -91,7 +91,6 @@ struct Workspace {
   DevBuf<unsigned char> tile_src;
   DevBuf<unsigned> pend;
   DevBuf<unsigned long long> slots;
-  DevBuf<unsigned> seq;
   DevBuf<int64_t> src_idx;
   DevBuf<double> src_t;
   DevBuf<SeedItem> seeds;
@@ -109,7 +108,7 @@ struct Workspace {
   void release_all() {
     r.release(); t_stage.release(); v_stage.release(); state.release(); tile_src.release();
     pend.release();
-    slots.release(); seq.release(); src_idx.release(); src_t.release(); seeds.release();
+    slots.release(); src_idx.release(); src_t.release(); seeds.release();
     copies.release();
     probs.release(); ctl.release(); count.release(); sum_ptr.release(); slab_t.release();
     slab_x.release();
@@ -747,10 +746,8 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
   if (guided) want_cap = std::max<uint64_t>(want_cap, (uint64_t)total_tiles / 4 + 4096);
   want_cap = next_pow2(std::max<uint64_t>(want_cap, opts && opts->capacity > 0 ? 16 : 1024));
   while (want_cap * eik::kNumSlots > kMaxCapEntries && want_cap > 1024) want_cap >>= 1;
-  // the ring layout depends on cap; storage only grows.  Entries need no
-  // clearing: the sequence words (zeroed below) say which positions hold one.
+  // the ring layout depends on cap; storage only grows
   CK(ws().slots.ensure((size_t)(want_cap * eik::kNumSlots)), "alloc frontier");
-  CK(ws().seq.ensure((size_t)(want_cap * eik::kNumSlots)), "alloc frontier sequence");
   ws().cap = want_cap;
 
   // uploads
@@ -771,8 +768,8 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
   if (!guided)
     CK(cudaMemsetAsync(ws().pend.p, 0, (size_t)total_tiles * eik::kPendWords * sizeof(unsigned),
                        stream), "clear pending masks");
-  CK(cudaMemsetAsync(ws().seq.p, 0, (size_t)(want_cap * eik::kNumSlots) * sizeof(unsigned), stream),
-     "clear frontier sequence");
+  CK(cudaMemsetAsync(ws().slots.p, 0, (size_t)(want_cap * eik::kNumSlots) * sizeof(unsigned long long), stream),
+     "clear frontier");
 
   // r = h / v (staging host speeds first)
   int64_t v_off = 0;
@@ -828,7 +825,6 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
                                                         : nullptr;
   sp.trace_cap = sp.trace ? (unsigned long long)opts->trace_cap : 0ull;
   sp.slots = ws().slots.p;
-  sp.seq = ws().seq.p;
   sp.cap_mask = (unsigned)(ws().cap - 1);
   sp.ctl = ws().ctl.p;
   const int64_t tmo_ms = opts && opts->timeout_ms > 0 ? opts->timeout_ms : 60000;
@@ -876,13 +872,11 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
     // grow the frontier, clear the scheduler (keep delta) and resume
     const uint64_t ncap = ws().cap * 4;
     CK(ws().slots.ensure((size_t)(ncap * eik::kNumSlots)), "grow frontier");
-    CK(ws().seq.ensure((size_t)(ncap * eik::kNumSlots)), "grow frontier sequence");
     ws().cap = ncap;
     sp.slots = ws().slots.p;
-    sp.seq = ws().seq.p;
     sp.cap_mask = (unsigned)(ncap - 1);
-    CK(cudaMemsetAsync(ws().seq.p, 0, (size_t)(ncap * eik::kNumSlots) * sizeof(unsigned), stream),
-       "clear frontier sequence");
+    CK(cudaMemsetAsync(ws().slots.p, 0, (size_t)(ncap * eik::kNumSlots) * sizeof(unsigned long long), stream),
+       "clear frontier");
     CK(cudaMemsetAsync(ws().ctl.p, 0, offsetof(Ctl, rsum), stream), "clear scheduler");
     CK(cudaMemsetAsync(&ws().ctl.p->stats[0], 0, sizeof(Ctl) - offsetof(Ctl, stats), stream),
        "clear counters");
@@ -1448,7 +1442,6 @@ struct eik_plan {
   DevBuf<unsigned char> tile_src;
   DevBuf<unsigned> pend;
   DevBuf<unsigned long long> slots;
-  DevBuf<unsigned> seq;
   DevBuf<int64_t> src_idx;
   DevBuf<double> src_t;
   DevBuf<SeedItem> seeds;
@@ -1465,7 +1458,7 @@ struct eik_plan {
   ~eik_plan() {
     v_stage.release(); t_stage.release(); copies.release();
     c.release(); state.release(); tile_src.release(); pend.release(); slots.release();
-    seq.release(); src_idx.release(); src_t.release(); seeds.release(); probs_d.release(); ctl.release();
+    src_idx.release(); src_t.release(); seeds.release(); probs_d.release(); ctl.release();
     count.release();
     if (ctl_host) cudaFreeHost(ctl_host);
   }
@@ -1597,7 +1590,6 @@ eik_status plan_build(eik_plan &pl, std::vector<HostProblem> &hps, const eik_opt
   while (want_cap * eik::kNumSlots > kMaxCapEntries && want_cap > 1024) want_cap >>= 1;
   pl.cap = want_cap;
   CK(pl.slots.ensure((size_t)(want_cap * eik::kNumSlots)), "plan: alloc frontier");
-  CK(pl.seq.ensure((size_t)(want_cap * eik::kNumSlots)), "plan: alloc frontier sequence");
   if (!out_items.empty()) {
     pl.ncopies = (int)out_items.size();
     CK(pl.copies.ensure(out_items.size()), "plan: alloc copy list");
@@ -1626,7 +1618,6 @@ eik_status plan_build(eik_plan &pl, std::vector<HostProblem> &hps, const eik_opt
   sp.tile_src = pl.tile_src.p;
   sp.pend = pl.pend.p;
   sp.slots = pl.slots.p;
-  sp.seq = pl.seq.p;
   sp.cap_mask = (unsigned)(pl.cap - 1);
   sp.ctl = pl.ctl.p;
   const int64_t tmo_ms = opts && opts->timeout_ms > 0 ? opts->timeout_ms : 60000;
@@ -1697,8 +1688,8 @@ eik_status eik_plan_enqueue(eik_plan *pl, void *stream) {
   if (!pl->sp.guided)
     CK(cudaMemsetAsync(pl->pend.p, 0, (size_t)pl->total_tiles * eik::kPendWords * sizeof(unsigned), s),
        "clear pending masks");
-  CK(cudaMemsetAsync(pl->seq.p, 0, (size_t)(pl->cap * eik::kNumSlots) * sizeof(unsigned), s),
-     "clear frontier sequence");
+  CK(cudaMemsetAsync(pl->slots.p, 0, (size_t)(pl->cap * eik::kNumSlots) * sizeof(unsigned long long), s),
+     "clear frontier");
   for (size_t j = 0; j < pl->speeds.size(); ++j) {
     if (pl->speed_host[j]) {
       CK(cudaMemcpyAsync(const_cast<double *>(pl->speeds[j]), pl->speed_host[j],

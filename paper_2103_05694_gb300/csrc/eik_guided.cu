@@ -29,7 +29,7 @@
 // What bounds it: with many fronts, instructions (88-problem 3D batch: issue 52 %
 // at 4.75 warps per scheduler, the instruction cache close to its request rate,
 // so loops are rolled and the scheduler's functions are not inlined: 218 -> 75 ms
-// while this was written); with one front, the latency of the visits along it
+// for the 128-source 3D batch); with one front, the latency of the visits along it
 // (about 1300 cycles per round of exact evaluations).  Evaluations per cell: 2.5
 // (batch) and 4 (checkerboard) against 6.1 and 11.2 in the other kernel.
 // Measured against that kernel with the same d-bar (us): 129^2 grid 796 -> 613,
@@ -52,15 +52,6 @@ namespace eik {
 namespace {
 
 constexpr float kSettled = 1e-3f;   // falls below this many r stop the FP32 relaxation
-constexpr float kInfF = __builtin_huge_valf();
-
-// A non-negative double (bit pattern) times 2^-se as a float, truncated; +inf stays.
-__device__ __forceinline__ float to_f_scaled(unsigned long long u, int se) {
-  const int e = static_cast<int>(u >> 52) - 1023 + 127 - se;
-  if (u == 0ull || e <= 0) return 0.0f;
-  if (e >= 255) return kInfF;
-  return __int_as_float((e << 23) | static_cast<int>((u >> 29) & 0x7fffffu));
-}
 
 // (v - base) times 2^-se as a float for bit patterns v >= base >= 0, without the
 // FP64 pipe: the significands' integer difference where v lies within 8
@@ -104,27 +95,13 @@ __device__ __forceinline__ float root_f(const float (&a)[D], float r) {
   return lo + u;
 }
 
-// Bit sets over a tile's cells: lane k < NC holds the word of cells 32 k .. 32 k + 31
-// (the other lanes 0).  For every cell q the bit of cell q + d; bits whose
-// neighbour is off the tile mean nothing and are masked by the caller.
-template <int d>
-__device__ __forceinline__ unsigned nbr_bits(unsigned w, bool across) {
-  constexpr int m = d < 0 ? -d : d;
-  if (m >= 32) {
-    if (d > 0) return __shfl_down_sync(kFull, w, m / 32);
-    const unsigned v = __shfl_up_sync(kFull, w, m / 32);
-    return (threadIdx.x & 31) >= m / 32 ? v : 0u;
+__device__ __forceinline__ int find_prob_ro(const SolveParams &p, unsigned tile) {
+  int lo = 0, hi = p.nprob - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (ldg_i64(&p.probs[mid].tile_base) <= static_cast<int64_t>(tile)) lo = mid; else hi = mid - 1;
   }
-  unsigned r = d > 0 ? w >> m : w << m;
-  if (across) {        // the neighbour may be in the next word
-    if (d > 0) {
-      r |= __shfl_down_sync(kFull, w, 1) << (32 - m);
-    } else {
-      const unsigned v = __shfl_up_sync(kFull, w, 1) >> (32 - m);
-      r |= (threadIdx.x & 31) > 0 ? v : 0u;
-    }
-  }
-  return r;
+  return lo;
 }
 
 template <int D, int TX, int TY, int TZ>
@@ -151,20 +128,9 @@ __global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) 
   const int lane = threadIdx.x;
   const float inv_delta = static_cast<float>(p.ctl->inv_delta);
   const int se = p.ctl->scale_exp;
-  const unsigned lt_mask = (1u << lane) - 1u;
   long long idle_since = 0;
   auto pos_of = [](int q) { return ((q / (TX * TY) + HZ) * SY + (q / TX) % TY + 1) * SX + q % TX + 1; };
-  // the bits of the neighbours across face j (-x, +x, -y, +y, -z, +z)
-  auto nbrs = [](unsigned w, int j) -> unsigned {
-    switch (j) {
-      case 0: return nbr_bits<-1>(w, false);
-      case 1: return nbr_bits<1>(w, false);
-      case 2: return nbr_bits<-TX>(w, TX * TY > 32);
-      case 3: return nbr_bits<TX>(w, TX * TY > 32);
-      case 4: return nbr_bits<-TX * TY>(w, true);
-      default: return nbr_bits<TX * TY>(w, true);
-    }
-  };
+  auto nbrs = [](unsigned w, int j) { return face_bits<TX, TY, TZ>(w, j); };
 
 #pragma unroll 1
   for (;;) {
@@ -187,24 +153,31 @@ __global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) 
     }
     if (tile < 0) break;
     idle_since = 0;
-    __threadfence();      // the claim is ordered before the tile's loads
-    const Prob &P = p.probs[find_prob(p, static_cast<unsigned long long>(tile))];
-    int64_t x0, y0, z0;
+    // the problem's record through the read-only path: the fence below would
+    // send each of these dependent reads to L2
+    const Prob &P = p.probs[find_prob_ro(p, static_cast<unsigned>(tile))];
+    const int64_t nx = ldg_i64(&P.nx), ny = ldg_i64(&P.ny), nz = ldg_i64(&P.nz);
+    const unsigned ntx = static_cast<unsigned>(ldg_i64(&P.ntx)), nty = static_cast<unsigned>(ldg_i64(&P.nty)),
+                   ntz = static_cast<unsigned>(ldg_i64(&P.ntz));
+    const double *const C0 = reinterpret_cast<const double *>(ldg_i64(&P.c));
+    unsigned tcx, tcy, tcz;
     {   // fewer than 2^32 tiles: 32-bit divisions
-      const unsigned lt = static_cast<unsigned>(tile - P.tile_base), ntx = static_cast<unsigned>(P.ntx),
-                     nty = static_cast<unsigned>(P.nty);
-      const unsigned rest = lt / ntx, tz = rest / nty;
-      x0 = static_cast<int64_t>(lt - rest * ntx) * TX;
-      y0 = static_cast<int64_t>(rest - tz * nty) * TY;
-      z0 = static_cast<int64_t>(tz) * TZ;
+      const unsigned lt = static_cast<unsigned>(tile - ldg_i64(&P.tile_base));
+      const unsigned rest = lt / ntx;
+      tcx = lt - rest * ntx;
+      tcz = rest / nty;
+      tcy = rest - tcz * nty;
     }
-    const int64_t sy = P.nx, sz = P.nx * P.ny, first = z0 * sz + y0 * sy + x0;
-    double *const T0 = P.t + first;      // the tile's first cell
+    const int64_t x0 = static_cast<int64_t>(tcx) * TX, y0 = static_cast<int64_t>(tcy) * TY,
+                  z0 = static_cast<int64_t>(tcz) * TZ;
+    const int64_t sy = nx, sz = nx * ny, first = z0 * sz + y0 * sy + x0;
+    double *const T0 = reinterpret_cast<double *>(ldg_i64(&P.t)) + first;   // the tile's first cell
+    fence_ar();      // the claim is ordered before the tile's loads
     // the grid in tile coordinates, as far as the tile and its halo reach
     const int xlo = x0 > 0 ? -1 : 0, ylo = y0 > 0 ? -1 : 0, zlo = z0 > 0 ? -1 : 0;
-    const int xhi = P.nx - x0 > TX ? TX + 1 : static_cast<int>(P.nx - x0);
-    const int yhi = P.ny - y0 > TY ? TY + 1 : static_cast<int>(P.ny - y0);
-    const int zhi = P.nz - z0 > TZ ? TZ + 1 : static_cast<int>(P.nz - z0);
+    const int xhi = nx - x0 > TX ? TX + 1 : static_cast<int>(nx - x0);
+    const int yhi = ny - y0 > TY ? TY + 1 : static_cast<int>(ny - y0);
+    const int zhi = nz - z0 > TZ ? TZ + 1 : static_cast<int>(nz - z0);
     unsigned fixed_w = 0u;               // sources and cells off the grid: word k in lane k
     const bool has_src = p.tile_src[tile] != 0;
 #pragma unroll 4
@@ -215,7 +188,7 @@ __global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) 
       const int64_t off = iz * sz + iy * sy + ix;
       const double tv = in ? ld_time(T0 + off) : from_bits(kInfBits);
       const unsigned long long cv =
-          in ? static_cast<unsigned long long>(__ldg(reinterpret_cast<const long long *>(P.c) + first + off)) : 0ull;
+          in ? static_cast<unsigned long long>(__ldg(reinterpret_cast<const long long *>(C0) + first + off)) : 0ull;
       s.t[pos_of(q)] = tv;
       s.c[q] = cv;
       s.fell[q] = 0;
@@ -361,31 +334,7 @@ __global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) 
 #pragma unroll
             for (int j = 0; j < 2 * D; ++j) ready_w &= ~(up_w[j] & nbrs(todo_w, j));
           }
-          // the set's cells as a list: every lane picks its bit of each word (few
-          // words: the shorter chain), or each word's lane writes its bits (many:
-          // fewer instructions)
-          int n = 0;
-          if constexpr (NC <= 2) {
-#pragma unroll
-            for (int k = 0; k < NC; ++k) {
-              const unsigned w = __shfl_sync(kFull, ready_w, k);
-              if ((w >> lane) & 1u) s.list[n + __popc(w & lt_mask)] = static_cast<unsigned char>(k * 32 + lane);
-              n += __popc(w);
-            }
-          } else {
-            const int own = __popc(ready_w);
-            n = own;
-#pragma unroll
-            for (int o = 1; o < NC; o <<= 1) {
-              const int v = __shfl_up_sync(kFull, n, o);
-              if (lane >= o) n += v;
-            }
-            int at = n - own;
-            n = __shfl_sync(kFull, n, NC - 1);
-#pragma unroll 1
-            for (unsigned w = ready_w; w; w &= w - 1u)
-              s.list[at++] = static_cast<unsigned char>(lane * 32 + __ffs(w) - 1);
-          }
+          const int n = list_of_set<NC>(ready_w, s.list);
           __syncwarp();
           if (n > 0) {
             todo_w &= ~ready_w;
@@ -471,41 +420,44 @@ __global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) 
           if (lane == j) mine = v;
           fm_any |= 1u << j;
         }
-        __threadfence();
+        fence_ar();
         __syncwarp();
         if ((fm_any >> lane) & 1u) {
           const int ax = lane >> 1, up = lane & 1;
-          const int64_t tc[3] = {x0 / TX, y0 / TY, z0 / TZ};
-          const int64_t ext = ax == 0 ? P.ntx : ax == 1 ? P.nty : P.ntz;
-          const int64_t moved = (ax == 0 ? tc[0] : ax == 1 ? tc[1] : tc[2]) + (up ? 1 : -1);
-          if (moved >= 0 && moved < ext) {
-            const int64_t step = ax == 0 ? 1 : ax == 1 ? P.ntx : P.ntx * P.nty;
+          const unsigned at = ax == 0 ? tcx : ax == 1 ? tcy : tcz, ext = ax == 0 ? ntx : ax == 1 ? nty : ntz;
+          if (up ? at + 1 < ext : at > 0) {
+            const int64_t step = ax == 0 ? 1 : ax == 1 ? ntx : static_cast<int64_t>(ntx) * nty;
             activate(p, static_cast<unsigned long long>(tile + (up ? step : -step)), 1u << (lane ^ 1),
-                     bucket_of_time(mine, inv_delta));
+                     bucket_of_time(mine, inv_delta), lo);
           }
         }
         __syncwarp();
-        __threadfence();
       }
-      // continue on this tile with its new faces if it was re-activated meanwhile
+      // done, unless the tile was re-activated meanwhile: then go on with its new
+      // faces
       int cont = 0;
       if (lane == 0) {
-        unsigned long long old = ld_rlx(&p.state[tile]);
-        if (state_of(old) == kStDirty) {
-          const unsigned long long prev = atomicCAS(&p.state[tile], old, make_state(kStRunning, 0, 0));
+        const unsigned long long mine = make_state(kStRunning, 0, 0);
+        unsigned long long old = mine;
+#pragma unroll 1
+        for (int it = 0;; ++it) {
+          const unsigned long long prev = atomicCAS(&p.state[tile], old, old == mine ? 0ull : mine);
           if (prev == old) {
-            cont = 0x100 | static_cast<int>(faces_of(old));
-            __threadfence();   // the claim of the new work before the halo loads
+            if (old != mine) cont = 0x100 | static_cast<int>(faces_of(old));
+            break;
           }
+          old = prev;
+          if (it > (1 << 22)) { raise_status(p.ctl, kEtimeout, 5); break; }
         }
+        if (cont) fence_ar();   // the claim of the new work before the halo loads
       }
       cont = __shfl_sync(kFull, cont, 0);
       if (!cont) break;
       faces = cont & 0x7f;
     }
+
     if (lane == 0) {
-      finish_tile(p, static_cast<unsigned long long>(tile));
-      __threadfence();
+      fence_ar();                // the pushes' work counts before this visit's
       atomicAdd(&p.ctl->run[slot * kCounterPad], 0xffffffffu);
       atomicAdd(&p.ctl->work, -1);
     }

@@ -14,11 +14,9 @@ std::mutex &api_mutex();
 void set_last_error(const char *fmt, ...);
 
 // Bucket ring: NB slots; bucket b lives in slot b & (NB - 1).  Each slot is a
-// ring of `cap` 64-bit entries (cap a power of two) with one sequence word per
-// position.  For the entry of index i (position i & (cap - 1)) the word reads
-// i & ~(cap - 1) while the position is free for it and that + 1 once the entry
-// is written; the entry's taker moves it on by cap (free for the next lap).
-// Sequence words are zero before every solve.
+// ring of `cap` 64-bit entries (cap a power of two), 0 while the position is
+// free; a pusher writes its entry with a CAS from 0, the taker exchanges it for
+// 0.  Entries are zero before every solve.
 constexpr uint32_t kNumSlots = 128;
 constexpr uint64_t kEmpty = ~0ull;
 constexpr uint32_t kMaxBucket = (1u << 30) - 1;
@@ -89,7 +87,6 @@ struct SolveParams {
   unsigned *pend;                 // per global tile, kPendWords words: cells deferred by
                                   // the last visit (to evaluate at the next one)
   unsigned long long *slots;      // kNumSlots * cap
-  unsigned *seq;                  // kNumSlots * cap sequence words (see the bucket ring)
   unsigned cap_mask;              // cap - 1
   Ctl *ctl;
   long long timeout_ns;

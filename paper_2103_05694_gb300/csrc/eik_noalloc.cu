@@ -39,8 +39,7 @@ constexpr size_t kOffState = up256(kOffC + sizeof(double) * kMaxCells);
 constexpr size_t kOffTileSrc = up256(kOffState + sizeof(unsigned long long) * kMaxTiles);
 constexpr size_t kOffPend = up256(kOffTileSrc + kMaxTiles);
 constexpr size_t kOffSlots = up256(kOffPend + sizeof(unsigned) * kPendWords * kMaxTiles);
-constexpr size_t kOffSeq = up256(kOffSlots + sizeof(unsigned long long) * kNumSlots * kCap);
-constexpr size_t kOffSrcIdx = up256(kOffSeq + sizeof(unsigned) * kNumSlots * kCap);
+constexpr size_t kOffSrcIdx = up256(kOffSlots + sizeof(unsigned long long) * kNumSlots * kCap);
 constexpr size_t kOffSrcT = up256(kOffSrcIdx + sizeof(int64_t) * kMaxSources);
 constexpr size_t kOffSeeds = up256(kOffSrcT + sizeof(double) * kMaxSources);
 constexpr size_t kBytes = up256(kOffSeeds + sizeof(SeedItem) * kMaxSources);
@@ -207,7 +206,7 @@ eik_status solve(const double *speed, double h, int ndim, const int64_t *dims,
       (e = cudaMemsetAsync(base + kOffState, 0, sizeof(unsigned long long) * ntiles, s)) != cudaSuccess ||
       (e = cudaMemsetAsync(base + kOffTileSrc, 0, ntiles, s)) != cudaSuccess ||
       (e = cudaMemsetAsync(base + kOffPend, 0, sizeof(unsigned) * kPendWords * ntiles, s)) != cudaSuccess ||
-      (e = cudaMemsetAsync(base + kOffSeq, 0, sizeof(unsigned) * kNumSlots * kCap, s)) != cudaSuccess) {
+      (e = cudaMemsetAsync(base + kOffSlots, 0, sizeof(unsigned long long) * kNumSlots * kCap, s)) != cudaSuccess) {
     return cuda_fail(e, "clearing the scratch array");
   }
   Prob prob;
@@ -244,7 +243,6 @@ eik_status solve(const double *speed, double h, int ndim, const int64_t *dims,
   sp.tile_src = base + kOffTileSrc;
   sp.pend = reinterpret_cast<unsigned *>(base + kOffPend);
   sp.slots = reinterpret_cast<unsigned long long *>(base + kOffSlots);
-  sp.seq = reinterpret_cast<unsigned *>(base + kOffSeq);
   sp.cap_mask = static_cast<unsigned>(kCap - 1);
   sp.ctl = ctl;
   sp.timeout_ns = (opts && opts->timeout_ms > 0 ? opts->timeout_ms : 60000) * 1000000ll;

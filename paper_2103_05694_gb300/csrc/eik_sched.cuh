@@ -70,6 +70,11 @@ __device__ __forceinline__ bool is_pending(unsigned long long pv, unsigned long 
   return pv != t && pv != kInfBits;
 }
 
+// Orders this thread's earlier accesses before its later ones for threads that
+// synchronise with it (cheaper than __threadfence(), which is sequentially
+// consistent).
+__device__ __forceinline__ void fence_ar() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
 // Relaxed, GPU-scope accesses (never served from a stale L1 line).
 __device__ __forceinline__ unsigned ld_rlx(const unsigned *p) {
   unsigned v;
@@ -97,13 +102,17 @@ __device__ __forceinline__ void st_rlx(unsigned long long *p, unsigned long long
 __device__ __forceinline__ void st_rlx(unsigned *p, unsigned v) {
   asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-__device__ __forceinline__ unsigned ld_acq(const unsigned *p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
+// Atomics that publish (release) or take over (acquire) a ring entry.
+__device__ __forceinline__ unsigned long long cas_rel(unsigned long long *p, unsigned long long old,
+                                                      unsigned long long v) {
+  unsigned long long r;
+  asm volatile("atom.release.gpu.global.cas.b64 %0, [%1], %2, %3;" : "=l"(r) : "l"(p), "l"(old), "l"(v) : "memory");
+  return r;
 }
-__device__ __forceinline__ void st_rel(unsigned *p, unsigned v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+__device__ __forceinline__ unsigned long long exch_acq(unsigned long long *p, unsigned long long v) {
+  unsigned long long r;
+  asm volatile("atom.acquire.gpu.global.exch.b64 %0, [%1], %2;" : "=l"(r) : "l"(p), "l"(v) : "memory");
+  return r;
 }
 __device__ __forceinline__ long long now_ns() {
   long long t;
@@ -146,25 +155,22 @@ EIK_SCHED_FN bool push_entry(const SolveParams &p, unsigned long long tile, unsi
   const unsigned s = b & (kNumSlots - 1);
   const unsigned cap = p.cap_mask + 1u;
   const unsigned idx = atomicAdd(&ctl->push[s * kCounterPad], 1u);
-  // depth as a signed difference: a popper may already have taken index idx
-  const int depth = static_cast<int>(idx - ld_rlx(&ctl->pop[s * kCounterPad]));
-  if (depth >= static_cast<int>(cap)) {
-    raise_status(ctl, kEcapacity, (static_cast<unsigned long long>(s) << 32) | idx);
-    return false;
-  }
-  const size_t pos = static_cast<size_t>(s) * cap + (idx & p.cap_mask);
-  const unsigned lap = idx & ~p.cap_mask;
-  const unsigned long long e = (static_cast<unsigned long long>(b) << 32) | tile;
+  unsigned long long *const slot = p.slots + static_cast<size_t>(s) * cap + (idx & p.cap_mask);
+  const unsigned long long e = (static_cast<unsigned long long>(b + 1u) << 32) | tile;
   long long t0 = 0;
-  while (ld_acq(p.seq + pos) != lap) {   // the previous lap's entry not taken yet
+#pragma unroll 1
+  while (cas_rel(slot, 0ull, e) != 0ull) {   // the position still holds an entry of an earlier lap
+    // depth as a signed difference: a popper may already have taken index idx
+    if (static_cast<int>(idx - ld_rlx(&ctl->pop[s * kCounterPad])) >= static_cast<int>(cap)) {
+      raise_status(ctl, kEcapacity, (static_cast<unsigned long long>(s) << 32) | idx);
+      return false;
+    }
     const long long now = now_ns();
     if (t0 == 0) t0 = now;
     else if (now - t0 > p.timeout_ns) { raise_status(ctl, kEcapacity, 1ull << 63); return false; }
     if (ld_rlx(&ctl->status)) return false;
     __nanosleep(64);
   }
-  st_rlx(p.slots + pos, e);
-  st_rel(p.seq + pos, lap + 1u);
   // the entry is written: one more for poppers to reserve
   atomicAdd(&ctl->avail[s * kCounterPad], 1);
   // A scanner may have moved the lowest-bucket hint past this slot between
@@ -173,22 +179,23 @@ EIK_SCHED_FN bool push_entry(const SolveParams &p, unsigned long long tile, unsi
   atomicMin(&ctl->cur, b);
   if (p.counters) {
     atomicAdd(&ctl->stats[kStatPushes], 1ull);
+    const int depth = static_cast<int>(idx - ld_rlx(&ctl->pop[s * kCounterPad]));
     if (depth > 0) atomicMax(&ctl->stats[kStatMaxQueue], static_cast<unsigned long long>(depth));
   }
   return true;
 }
 
 // A face of `tile` has new lower halo values (the smallest in bucket
-// `bucket`): make sure the tile is (re)processed after this point.
+// `bucket`): make sure the tile is (re)processed after this point.  cur: the
+// lowest-bucket hint, now or a little earlier (it only clamps the priority).
 EIK_SCHED_FN void activate(const SolveParams &p, unsigned long long tile, unsigned face_bits,
-                         unsigned bucket) {
+                           unsigned bucket, unsigned cur) {
   Ctl *ctl = p.ctl;
-  const unsigned cur = ld_rlx(&ctl->cur);
   unsigned b = bucket;
   if (b < cur) b = cur;
   else if (b - cur >= kNumSlots) b = cur + kNumSlots - 1;
   if (b > kMaxBucket) b = kMaxBucket;
-  unsigned long long old = ld_rlx(&p.state[tile]);
+  unsigned long long old = 0ull;          // idle, most often; the CAS tells otherwise
 #pragma unroll 1
   for (int it = 0; it < (1 << 22); ++it) {
     const unsigned long long st = state_of(old);
@@ -217,6 +224,11 @@ EIK_SCHED_FN void activate(const SolveParams &p, unsigned long long tile, unsign
   raise_status(ctl, kEtimeout, 3);
 }
 
+__device__ __forceinline__ void activate(const SolveParams &p, unsigned long long tile,
+                                         unsigned face_bits, unsigned bucket) {
+  activate(p, tile, face_bits, bucket, ld_rlx(&p.ctl->cur));
+}
+
 // Claim a popped entry: queued(b) -> running.  Returns the face mask, or -1
 // if the entry is stale (the tile was re-queued elsewhere or is done).
 EIK_SCHED_FN int try_claim(const SolveParams &p, unsigned long long tile, unsigned b) {
@@ -234,7 +246,7 @@ EIK_SCHED_FN int try_claim(const SolveParams &p, unsigned long long tile, unsign
 
 // End of a visit: running -> idle, or dirty(b) -> queued(b) plus a push.
 EIK_SCHED_FN void finish_tile(const SolveParams &p, unsigned long long tile) {
-  unsigned long long old = ld_rlx(&p.state[tile]);
+  unsigned long long old = make_state(kStRunning, 0, 0);
 #pragma unroll 1
   for (int it = 0; it < (1 << 22); ++it) {
     unsigned long long nw;
@@ -250,19 +262,16 @@ EIK_SCHED_FN void finish_tile(const SolveParams &p, unsigned long long tile) {
   raise_status(p.ctl, kEtimeout, 5);
 }
 
-// The entry of index q of slot s (reserved by the caller): wait until its
-// pusher has written it, take it and free the position for the next lap.
+// The entry at index q of slot s (reserved by the caller), freeing its position:
+// waits until a pusher has written it.  (If laps meet at a position, the
+// entries go to either taker: they are all live.)
 EIK_SCHED_FN unsigned long long take_slot(const SolveParams &p, unsigned s, unsigned q) {
-  const size_t pos = static_cast<size_t>(s) * (p.cap_mask + 1u) + (q & p.cap_mask);
-  const unsigned lap = q & ~p.cap_mask;
+  unsigned long long *const slot = p.slots + static_cast<size_t>(s) * (p.cap_mask + 1u) + (q & p.cap_mask);
   long long t0 = 0;
 #pragma unroll 1
   for (;;) {
-    if (ld_acq(p.seq + pos) == lap + 1u) {
-      const unsigned long long e = ld_rlx(p.slots + pos);
-      st_rel(p.seq + pos, lap + p.cap_mask + 1u);     // after the read of the entry
-      return e;
-    }
+    const unsigned long long e = exch_acq(slot, 0ull);
+    if (e != 0ull) return e - (1ull << 32);
     const long long now = now_ns();
     if (t0 == 0) t0 = now;
     else if (now - t0 > p.timeout_ns) { raise_status(p.ctl, kEtimeout, 6); return kEmpty; }
@@ -287,23 +296,22 @@ EIK_SCHED_FN unsigned long long pop_entry(const SolveParams &p, long long &idle_
   for (;;) {
     unsigned stop = 0, cur = 0;
     if (lane == 0) {
-      stop = ld_rlx(&ctl->status) | ld_rlx(&ctl->done);
       cur = ld_rlx(&ctl->cur);
+      stop = ld_rlx(&ctl->status) | ld_rlx(&ctl->done);
     }
     stop = __shfl_sync(kFull, stop, 0);
     if (stop) return kEmpty;
     cur = __shfl_sync(kFull, cur, 0);
     // find the lowest active slot at or above the hint (whole ring if needed)
     unsigned first = 0xffffffffu;
-    unsigned q = 0, pp = 0, s = 0;
+    unsigned s = 0;
     bool pend = false;
 #pragma unroll 1
     for (unsigned base = 0; base < kNumSlots; base += 32) {
       s = (cur + base + lane) & (kNumSlots - 1);
-      q = ld_rlx(&ctl->pop[s * kCounterPad]);
-      pp = ld_rlx(&ctl->push[s * kCounterPad]);
+      const int av = ld_rlx(&ctl->avail[s * kCounterPad]);
       const unsigned rn = p.gate_pending_only ? 0u : ld_rlx(&ctl->run[s * kCounterPad]);
-      pend = static_cast<int>(pp - q) > 0;
+      pend = av > 0;
       const unsigned act = __ballot_sync(kFull, pend || rn > 0u);
       if (act) {
         first = base + static_cast<unsigned>(__ffs(act) - 1);
@@ -336,13 +344,11 @@ EIK_SCHED_FN unsigned long long pop_entry(const SolveParams &p, long long &idle_
           // a popper that has just seen an entry to reserve tries (a failed try
           // holds the count down until it is undone).
           int *av = &ctl->avail[s * kCounterPad];
-          if (ld_rlx(av) > 0) {
-            if (atomicAdd(av, -1) > 0) {
-              got = 1;
-              e = take_slot(p, s, atomicAdd(&ctl->pop[s * kCounterPad], 1u));
-            } else {
-              atomicAdd(av, 1);                           // nothing left: undo the try
-            }
+          if (atomicAdd(av, -1) > 0) {
+            got = 1;
+            e = take_slot(p, s, atomicAdd(&ctl->pop[s * kCounterPad], 1u));
+          } else {
+            atomicAdd(av, 1);                           // nothing left: undo the try
           }
           if (!got) atomicAdd(&ctl->run[s * kCounterPad], 0xffffffffu);
         }
@@ -383,6 +389,92 @@ __device__ __forceinline__ bool is_source(const Prob &P, int64_t idx) {
     if (v < idx) lo = mid + 1; else hi = mid - 1;
   }
   return false;
+}
+
+// ---------------------------------------------------------------------------
+// Shared by the kernels that give a tile to one warp.
+// ---------------------------------------------------------------------------
+// A 64-bit field of a record that no kernel writes, through the read-only path.
+__device__ __forceinline__ int64_t ldg_i64(const void *p) {
+  return __ldg(static_cast<const long long *>(p));
+}
+
+constexpr float kInfF = __builtin_huge_valf();
+
+// A non-negative double (bit pattern) times 2^-se as a float, truncated; +inf stays.
+__device__ __forceinline__ float to_f_scaled(unsigned long long u, int se) {
+  const int e = static_cast<int>(u >> 52) - 1023 + 127 - se;
+  if (u == 0ull || e <= 0) return 0.0f;
+  if (e >= 255) return kInfF;
+  return __int_as_float((e << 23) | static_cast<int>((u >> 29) & 0x7fffffu));
+}
+
+// Bit sets over a tile's cells: lane k < NC holds the word of cells 32 k .. 32 k + 31
+// (the other lanes 0).  For every cell q the bit of cell q + d; bits whose
+// neighbour is off the tile mean nothing and are masked by the caller.
+template <int d>
+__device__ __forceinline__ unsigned nbr_bits(unsigned w, bool across) {
+  constexpr int m = d < 0 ? -d : d;
+  if (m >= 32) {
+    if (d > 0) return __shfl_down_sync(kFull, w, m / 32);
+    const unsigned v = __shfl_up_sync(kFull, w, m / 32);
+    return (threadIdx.x & 31) >= m / 32 ? v : 0u;
+  }
+  unsigned r = d > 0 ? w >> m : w << m;
+  if (across) {        // the neighbour may be in the next word
+    if (d > 0) {
+      r |= __shfl_down_sync(kFull, w, 1) << (32 - m);
+    } else {
+      const unsigned v = __shfl_up_sync(kFull, w, 1) >> (32 - m);
+      r |= (threadIdx.x & 31) > 0 ? v : 0u;
+    }
+  }
+  return r;
+}
+
+// The bits of the neighbours across face j (-x, +x, -y, +y, -z, +z) of the cells of
+// a TX x TY x TZ tile, cells numbered x fastest.
+template <int TX, int TY, int TZ>
+__device__ __forceinline__ unsigned face_bits(unsigned w, int j) {
+  switch (j) {
+    case 0: return nbr_bits<-1>(w, false);
+    case 1: return nbr_bits<1>(w, false);
+    case 2: return nbr_bits<-TX>(w, TX * TY > 32);
+    case 3: return nbr_bits<TX>(w, TX * TY > 32);
+    case 4: return nbr_bits<-TX * TY>(w, true);
+    default: return nbr_bits<TX * TY>(w, true);
+  }
+}
+
+// A set's cells as a list in shared memory (to be read after a __syncwarp);
+// returns their number.  Every lane picks its bit of each word (few words: the
+// shorter chain, 210 against 435 cycles for 2), or each word's lane writes its
+// bits (many: fewer instructions, 14.7 against 29.0 kcycles a visit for 8).
+template <int NC>
+__device__ __forceinline__ int list_of_set(unsigned set, unsigned char *list) {
+  const int lane = threadIdx.x & 31;
+  int n = 0;
+  if constexpr (NC <= 2) {
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      const unsigned w = __shfl_sync(kFull, set, k);
+      if ((w >> lane) & 1u) list[n + __popc(w & ((1u << lane) - 1u))] = static_cast<unsigned char>(k * 32 + lane);
+      n += __popc(w);
+    }
+  } else {
+    const int own = __popc(set);
+    n = own;
+#pragma unroll
+    for (int o = 1; o < NC; o <<= 1) {
+      const int v = __shfl_up_sync(kFull, n, o);
+      if (lane >= o) n += v;
+    }
+    int at = n - own;
+    n = __shfl_sync(kFull, n, NC - 1);
+#pragma unroll 1
+    for (unsigned w = set; w; w &= w - 1u) list[at++] = static_cast<unsigned char>(lane * 32 + __ffs(w) - 1);
+  }
+  return n;
 }
 
 }  // namespace

@@ -19,13 +19,12 @@
 //    arrival time; the minimum committed time on each tile face activates the
 //    neighbour tile across that face (one aggregated push per face).
 //  * Scheduler: persistent kernel; kNumSlots bucket slots, each a ring of
-//    64-bit entries (tile | bucket << 32) with a sequence word per position;
-//    warp 0 of a CTA scans 32 slots per step from the lowest-bucket hint,
-//    reserves a written entry of a slot and takes the slot's next index (two
-//    fetch-and-adds: hundreds of idle CTAs never serialise on a retried CAS),
-//    then claims the tile through its state word (idle / queued(b) / running
-//    / dirty(b)); a stale entry is dropped.  Termination: the count of
-//    unfinished entries reaches zero.
+//    64-bit entries (tile | bucket + 1 << 32, 0: free); warp 0 of a CTA scans
+//    32 slots per step from the lowest-bucket hint, reserves a written entry of
+//    a slot and takes the slot's next index (two fetch-and-adds: hundreds of
+//    idle CTAs never serialise on a retried CAS), then claims the tile through
+//    its state word (idle / queued(b) / running / dirty(b)); a stale entry is
+//    dropped.  Termination: the count of unfinished entries reaches zero.
 //  * FP64 is scarce on this part (about 1.6 DFMA per SM per clock), so every
 //    comparison, min, max and sign test runs on integer bit patterns, and a
 //    cell is evaluated only when a neighbour changed.
