@@ -15,15 +15,15 @@
 // Set-up (fully parallel) evaluates everything that does not depend on lambda:
 // per cell m the mask of its upwind sides, the weight of each active axis
 // W_k(m) = fl(fl(t_m - a_k) / S_m) (halved on a tie) and the coefficient
-// fl(fl(h^2 fl(1 / v)) / S), and counts for every cell the downwind cells that
-// use it.  The dependent part is then one multiply-add per downwind neighbour.
+// fl(fl(h^2 fl(1 / v)) / S).  The dependent part is then one multiply-add per
+// downwind neighbour.
 //
 // Two schedules process the cells in dependency (Kahn) order with the same
 // operations in the same order, so their results are identical:
-//  * tiles (the default; see "Tile schedule" below): persistent CTAs take
-//    tiles from a queue and run the order inside a tile in shared memory,
-//    handing cross-tile dependencies over through counts and the queue;
-//  * levels: cells with count 0 form the first frontier; one cooperative
+//  * tiles (the default; see "Tile schedule" below): persistent warps take
+//    tiles from the bucket scheduler and run the order inside a tile in shared
+//    memory, handing cross-tile dependencies over through the cells' mask bytes;
+//  * levels: the set-up also counts every cell's downwind users; cells with count 0 form the first frontier; one cooperative
 //    persistent launch processes a frontier (each cell pulls lambda from its
 //    downwind cells, writes lambda and dL/ds, decrements its upwind cells'
 //    counts and appends those that reach zero to the next frontier), then its
@@ -34,8 +34,11 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "eik_exact.cuh"
 #include "eik_grid.cuh"
 #include "eik_internal.h"
+#define EIK_SCHED_FN __device__ __noinline__
+#include "eik_sched.cuh"
 
 namespace eik {
 namespace {
@@ -122,68 +125,117 @@ __device__ __forceinline__ int64_t nbr(const AdjProb &P, const Cell &e, int j) {
   return e.c[k] > 0 ? e.n - st : -1;
 }
 
-// Per cell: zeroed lambda, the upwind-side mask, per-axis weights, the gradient
-// coefficient (kept in grad until lambda is known), reached count, and the
-// downwind-use counts of the upwind cells.
-__global__ void adj_setup_kernel(const AdjProb *probs, int nprob, int64_t total, AdjCtl *ctl,
-                                 int tx, int ty, int tz) {
-  // tx > 0: tile schedule with tiles tx x ty x tz: a downwind user in another
-  // tile counts in cnt_out
-  const int tdim[3] = {tx, ty, tz};
+// Per cell: the upwind-side mask, per-axis weights, and the gradient coefficient
+// (kept in grad until lambda is known).
+constexpr unsigned kPending = 0x40u, kDone = 0x80u;   // tile schedule: in the mask byte
+
+// fl(h^2 s) of a cell, s = fl(1/v); slowness input: v = fl(1/s_in) as the forward used.
+__device__ __forceinline__ double h2s(double v, int v_is_slowness, double hh) {
+  const double vn = v_is_slowness ? ig::quotient(1.0, v) : v;
+  return __dmul_rn(hh, ig::quotient(1.0, vn));
+}
+
+// The same for a whole model that several problems share: the set-up is bound
+// by its divisions, of which a slowness model needs two here, and per problem one
+// per active axis and one for the coefficient.  32 problems of 1024^2 cells on one
+// model: set-up and this kernel 2.70 -> 1.9 ms by sharing (and a grid row per
+// problem in place of a search per cell), 1.02 ms with the divisions off the FP64
+// pipe (ig::Divisor).
+__global__ void adj_h2s_kernel(const double *__restrict__ v, int v_is_slowness, double hh, int64_t n,
+                               double *__restrict__ hs) {
+  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
+       i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+    hs[i] = h2s(v[i], v_is_slowness, hh);
+}
+
+// Mask, weights and coefficient of cell n with time tn; returns the mask.
+template <bool COUNT>
+__device__ __forceinline__ unsigned setup_cell(const AdjProb &P, int64_t n, double tn) {
+  double coef = 0.0;
+  unsigned mask = 0u;
+  if (ubits(tn) < kInfB && !(P.nsrc > 0 && adj_is_source(P, n))) {
+    const Cell e = cell_of(P, n);
+    unsigned long long lo[3], hi[3], ak[3];
+    double d[3], S = 0.0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (k >= P.ndim) break;
+      const int64_t a = nbr(P, e, 2 * k), b = nbr(P, e, 2 * k + 1);
+      lo[k] = a >= 0 ? ubits(P.t[a]) : kInfB;
+      hi[k] = b >= 0 ? ubits(P.t[b]) : kInfB;
+      ak[k] = lo[k] < hi[k] ? lo[k] : hi[k];
+      if (ak[k] < ubits(tn)) {
+        d[k] = __dsub_rn(tn, __longlong_as_double(static_cast<long long>(ak[k])));
+        S = __dadd_rn(S, d[k]);
+      }
+    }
+    if (S > 0.0) {   // else unreachable for a reached non-source cell
+      const ig::Divisor by_S(ubits(S));
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        if (k >= P.ndim) break;
+        if (!(ak[k] < ubits(tn))) continue;               // axis not active
+        double w = __longlong_as_double(static_cast<long long>(by_S.quotient(ubits(d[k]))));
+        if (lo[k] == hi[k]) w = __dmul_rn(w, 0.5);        // tie: half to each side
+        P.W[k][n] = w;
+        if (lo[k] == ak[k]) mask |= 1u << (2 * k);
+        if (hi[k] == ak[k]) mask |= 1u << (2 * k + 1);
+        if (COUNT) {
+          if (lo[k] == ak[k]) atomicAdd(P.cnt + nbr(P, e, 2 * k), 1);
+          if (hi[k] == ak[k]) atomicAdd(P.cnt + nbr(P, e, 2 * k + 1), 1);
+        }
+      }
+      coef = __longlong_as_double(static_cast<long long>(
+          by_S.quotient(ubits(P.hs ? P.hs[n] : h2s(P.v[n], P.v_is_slowness, P.hh)))));
+    }
+  }
+  P.grad[n] = coef;
+  return mask;
+}
+
+// Level schedule: also zeroed lambda and the downwind-use counts of the upwind cells.
+__global__ void adj_setup_kernel(const AdjProb *probs, int nprob, int64_t total, AdjCtl *ctl) {
   unsigned long long reached = 0;
   for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < total;
        q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const AdjProb &P = probs[find_adj_prob(probs, nprob, q)];
     const int64_t n = q - P.base;
-    if (P.lam) P.lam[n] = 0.0;   // the tile schedule does not store lambda
-    P.grad[n] = 0.0;
-    P.mask[n] = 0;
     const double tn = P.t[n];
-    const bool is_reached = ubits(tn) < kInfB;
-    if (tx > 0) P.status[n] = is_reached ? 1 : 0;
-    if (!is_reached) continue;
-    ++reached;
-    if (P.nsrc > 0 && adj_is_source(P, n)) continue;
-    const Cell e = cell_of(P, n);
-    unsigned long long lo[3], hi[3], ak[3];
-    double S = 0.0;
-    for (int k = 0; k < P.ndim; ++k) {
-      const int64_t a = nbr(P, e, 2 * k), b = nbr(P, e, 2 * k + 1);
-      lo[k] = a >= 0 ? ubits(P.t[a]) : kInfB;
-      hi[k] = b >= 0 ? ubits(P.t[b]) : kInfB;
-      ak[k] = lo[k] < hi[k] ? lo[k] : hi[k];
-      if (ak[k] < ubits(tn))
-        S = __dadd_rn(S, __dsub_rn(tn, __longlong_as_double(static_cast<long long>(ak[k]))));
-    }
-    if (!(S > 0.0)) continue;   // unreachable for a reached non-source cell
-    unsigned char mask = 0;
-    for (int k = 0; k < P.ndim; ++k) {
-      if (!(ak[k] < ubits(tn))) continue;               // axis not active
-      double w = __ddiv_rn(__dsub_rn(tn, __longlong_as_double(static_cast<long long>(ak[k]))), S);
-      if (lo[k] == hi[k]) w = __dmul_rn(w, 0.5);        // tie: half to each side
-      P.W[k][n] = w;
-      // the upwind neighbour on the low side is in another tile when this cell
-      // starts its tile along axis k; on the high side when it ends it
-      const bool lo_out = tx > 0 && e.c[k] % tdim[k] == 0;
-      const bool hi_out = tx > 0 && (e.c[k] + 1) % tdim[k] == 0;
-      if (lo[k] == ak[k]) {
-        mask |= static_cast<unsigned char>(1u << (2 * k));
-        atomicAdd((lo_out ? P.cnt_out : P.cnt) + nbr(P, e, 2 * k), 1);
-      }
-      if (hi[k] == ak[k]) {
-        mask |= static_cast<unsigned char>(1u << (2 * k + 1));
-        atomicAdd((hi_out ? P.cnt_out : P.cnt) + nbr(P, e, 2 * k + 1), 1);
-      }
-    }
-    P.mask[n] = mask;
-    // slowness input: v = fl(1/s_in) as the forward used, then s = fl(1/v)
-    const double vn = P.v_is_slowness ? __ddiv_rn(1.0, P.v[n]) : P.v[n];
-    const double s = __ddiv_rn(1.0, vn);
-    P.grad[n] = __ddiv_rn(__dmul_rn(P.hh, s), S);
+    reached += ubits(tn) < kInfB ? 1u : 0u;
+    P.lam[n] = 0.0;
+    P.mask[n] = static_cast<unsigned char>(setup_cell<true>(P, n, tn));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) reached += __shfl_xor_sync(kFullMask, reached, o);
   if ((threadIdx.x & 31) == 0 && reached) atomicAdd(&ctl->reached, reached);
+}
+
+// Tile schedule: the mask byte carries kPending (reached), and the problem's
+// largest time is collected (the tiles' order).  blockIdx.y: problem (first + y),
+// so that no cell searches for its problem and a warp needs one atomic.
+__global__ void adj_setup_tiles_kernel(const AdjProb *probs, int first, AdjCtl *ctl) {
+  const AdjProb &P = probs[first + blockIdx.y];
+  const int64_t total = P.nx * P.ny * P.nz;
+  unsigned long long reached = 0;
+  unsigned top = 0u;        // high word of the largest finite time
+  for (int64_t n = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; n < total;
+       n += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    const double tn = P.t[n];
+    const bool is_reached = ubits(tn) < kInfB;
+    if (is_reached) {
+      ++reached;
+      const unsigned hi = static_cast<unsigned>(ubits(tn) >> 32);
+      top = top < hi ? hi : top;
+    }
+    P.mask[n] = static_cast<unsigned char>(setup_cell<false>(P, n, tn) | (is_reached ? kPending : 0u));
+  }
+  top = __reduce_max_sync(kFullMask, top);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) reached += __shfl_xor_sync(kFullMask, reached, o);
+  if ((threadIdx.x & 31) == 0) {
+    if (reached) atomicAdd(&ctl->reached, reached);
+    if (top) atomicMax(P.tmax, static_cast<unsigned long long>(top) << 32);
+  }
 }
 
 // Warp-aggregated append of the lanes' ready entries to a frontier.  All 32
@@ -298,442 +350,359 @@ __global__ void __launch_bounds__(kThreads) adj_levels_kernel(const AdjProb *pro
 }
 
 // ---------------------------------------------------------------------------
-// Tile schedule.  The same per-cell work in the same order as above, but the
-// unit of scheduling is a tile of cells held in shared memory.  A cell's users
-// are split into those in its own tile (cnt, decremented in shared memory while
-// the tile is visited) and those in other tiles (cnt_out, decremented with a
-// global atomic after the user's lambda is published).  A tile is visited when
-// one of its cells may have become ready; a visit runs Kahn rounds in shared
-// memory until none of its cells is ready, so the critical path costs a block
-// barrier per level instead of a grid barrier.
+// Tile schedule.  The same per-cell work in the same order as above; the unit
+// of scheduling is a tile, given to one warp.  A cell n is ready when every
+// downwind user of it (a neighbour m whose mask names n's side) is done.  A visit
+// loads the tile and the mask bytes around it: cells with a user across the
+// tile edge that is not done are blocked for this visit, the others are
+// processed in dependency order, kept as bit sets over the tile (one word per
+// lane, as in the forward kernel): ready cells are those none of whose in-tile
+// users is left, packed onto the lanes.  Each sums g and the products of its
+// users in the fixed order (x-, x+, y-, y+, z-, z+) and turns its weights W_k
+// into products p_k = fl(lambda W_k), which is all its upwind cells need.  Then
+// the tile's gradients are written, the products that another tile or a later
+// visit reads, after a fence the mask bytes with kDone, and the tiles that hold
+// upwind cells of this tile's are activated.
 //
-// Tile state word: bit 0 = activated (queued, or to be queued again), bit 1 =
-// being visited.  Activation is one atomicOr, so it is ordered against the
-// visitor's claim and finish.  The queue is a bounded ring of sequence-tagged
-// slots: a slot holds FREE(i) when index i may be pushed into it, FULL(i, tile)
-// once pushed.
+// The forward solver's bucket scheduler orders the tiles by decreasing time (of
+// the cell in the tile's middle, in fractions of the problem's largest time), so
+// that a tile's users are mostly done when it is taken.
+//
+// What bounds it: the chain of tiles (a visit is about 40 kcycles, of which the
+// loads and the stores take three quarters), so many small tiles in flight count,
+// and few visits per tile.  Against per-cell counts (two arrays, atomics in the
+// set-up and at every release), a FIFO of tiles and a block of 128 (2D) or 256
+// threads per tile with a barrier per round: 8.97 -> 4.97 ms for 32 problems of
+// 1024^2 cells, 6.6 -> 3.6 ms for one of 192 x 224 x 208.  Tiles: 16x16 in 2D
+// (16x8 and 8x8: 9.8 and 10.5 ms against 8.9 for set-up and tiles), 8x4x4 in 3D
+// (8x8x4 and 4x4x4: 4.7 and 4.9 against 4.5).  12 warps per SM (20 are slower:
+// 10.4 and 6.2 ms; the tiles wait for each other, not for a warp).  Steps of the
+// order: 0.04 (nx + ny + nz) per field in 2D (0.25: 11.2 ms, 0.1: 10.2, none:
+// 10.1, against 9.8), 0.15 in 3D (0.25: 4.90, 0.04: 4.95, none: 6.3, against 4.85).
 // ---------------------------------------------------------------------------
-constexpr unsigned kTActive = 1u, kTRunning = 2u;
-constexpr unsigned kNoTile = 0xffffffffu;
+template <int D, int TX, int TY, int TZ>
+struct ATile {
+  static constexpr int NT = TX * TY * TZ, NC = NT / 32;
+  static constexpr int HZ = D == 3 ? 1 : 0;
+  static constexpr int SX = TX + 2, SY = TY + 2, SZ = TZ + 2 * HZ, NS = SX * SY * SZ;
+  double p[D][NS];                 // W_k, p_k once done (halo: p_k of the axis across the face)
+  double lam[NT];                  // g, lambda once done
+  unsigned char m[NS];             // mask bytes with halo
+  unsigned char list[NT];
+};
 
-__device__ __forceinline__ unsigned long long slot_free(unsigned long long i) {
-  return (i << 32) | kNoTile;
-}
-__device__ __forceinline__ unsigned long long slot_full(unsigned long long i, unsigned tile) {
-  return (i << 32) | tile;
-}
-__device__ __forceinline__ unsigned long long ld_rlx_slot(const unsigned long long *p) {
-  return ld_rlx_u64(p);
-}
-__device__ __forceinline__ void st_rlx_u64(unsigned long long *p, unsigned long long v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ int ld_acq_s32(const int *p) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ int ld_rlx_s32(const int *p) {
-  int v;
-  asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
 __device__ __forceinline__ unsigned ld_rlx_u8(const unsigned char *p) {
   unsigned short v;
   asm volatile("ld.relaxed.gpu.global.u8 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
   return v;
 }
 
-struct TileQueue {
-  unsigned *state;
-  unsigned long long *ring;
-  unsigned long long mask;   // ring slots - 1
-  AdjCtl *ctl;
-  long long timeout_ns;
-};
-
-__device__ __forceinline__ void tq_fail(const TileQueue &q) { atomicCAS(&q.ctl->status, 0u, kEtimeout); }
-
-__device__ void tq_push(const TileQueue &q, unsigned tile) {
-  const unsigned long long i = atomicAdd(&q.ctl->tail, 1ull);
-  unsigned long long *slot = q.ring + (i & q.mask);
-  const long long t0 = grid::now_ns();
-  // at most total_tiles tiles are queued and the ring has at least that many
-  // slots, so the slot's previous index has a taker, which frees it
-  while (ld_rlx_slot(slot) != slot_free(i & 0xffffffffull)) {
-    if (grid::now_ns() - t0 > q.timeout_ns) { tq_fail(q); return; }
-  }
-  st_rlx_u64(slot, slot_full(i & 0xffffffffull, tile));
-}
-
-// A cell of `tile` may have become ready (called after the release it follows
-// and a fence).
-__device__ void tq_activate(const TileQueue &q, unsigned tile) {
-  if (atomicOr(q.state + tile, kTActive) == 0u) tq_push(q, tile);   // was idle
-}
-
-// Take the next queued tile; -1 when every reached cell is done or on error.
-// The taker draws a ticket (fetch-and-add, no retry under contention) and
-// waits on that slot alone until its tile is pushed.  The wait gives up when
-// no cell has been processed anywhere for timeout_ns.
-__device__ long long tq_pop(const TileQueue &q, unsigned long long reached) {
-  const unsigned long long h = atomicAdd(&q.ctl->head, 1ull);
-  unsigned long long *slot = q.ring + (h & q.mask);
-  const unsigned long long tag = (h & 0xffffffffull) << 32;
-  unsigned long long last_done = ~0ull;
-  long long since = 0;
-#pragma unroll 1
-  for (;;) {
-    const unsigned long long v = ld_rlx_slot(slot);
-    if ((v & ~0xffffffffull) == tag && static_cast<unsigned>(v) != kNoTile) {
-      st_rlx_u64(slot, slot_free((h + q.mask + 1ull) & 0xffffffffull));
-      return static_cast<long long>(static_cast<unsigned>(v));
-    }
-    if (grid::ld_acq(&q.ctl->status) != 0u) return -1;
-    const unsigned long long d = ld_rlx_u64(&q.ctl->done);
-    if (d >= reached) return -1;
-    const long long now = grid::now_ns();
-    if (d != last_done) {
-      last_done = d;
-      since = now;
-    } else if (now - since > q.timeout_ns) {
-      tq_fail(q);
-      return -1;
-    }
-    __nanosleep(128);
-  }
-}
-
-__device__ __forceinline__ int find_tile_prob(const AdjProb *probs, int nprob, long long tile) {
+__device__ __forceinline__ int find_tile_prob(const AdjProb *probs, int nprob, unsigned tile) {
   int lo = 0, hi = nprob - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (probs[mid].tile_base <= tile) lo = mid; else hi = mid - 1;
+    if (static_cast<unsigned long long>(ldg_i64(&probs[mid].tile_base)) <= tile) lo = mid; else hi = mid - 1;
   }
   return lo;
 }
 
+// Bucket of tile (tx, ty, tz) of P: how far its middle cell lies below the
+// problem's largest time, in steps of about two cells.
 template <int TX, int TY, int TZ>
-__device__ __forceinline__ unsigned tile_of_cell(const AdjProb &P, int64_t x, int64_t y, int64_t z) {
-  return static_cast<unsigned>(P.tile_base + ((z / TZ) * P.nty + (y / TY)) * P.ntx + (x / TX));
+__device__ __forceinline__ unsigned tile_bucket(const AdjProb &P, unsigned tx, unsigned ty, unsigned tz) {
+  const int64_t nx = ldg_i64(&P.nx), ny = ldg_i64(&P.ny), nz = ldg_i64(&P.nz);
+  const int64_t mx = static_cast<int64_t>(tx) * TX + TX / 2, my = static_cast<int64_t>(ty) * TY + TY / 2,
+                mz = static_cast<int64_t>(tz) * TZ + TZ / 2;
+  const int64_t x = mx < nx ? mx : nx - 1, y = my < ny ? my : ny - 1, z = mz < nz ? mz : nz - 1;
+  const double *const t = reinterpret_cast<const double *>(ldg_i64(&P.t));
+  const unsigned long long tb = static_cast<unsigned long long>(ldg_i64(t + (z * ny + y) * nx + x)),
+                           top = static_cast<unsigned long long>(ldg_i64(reinterpret_cast<const void *>(ldg_i64(&P.tmax))));
+  const int se = static_cast<int>(top >> 52) - 1023;
+  const float f = to_f_scaled(tb, se), ft = to_f_scaled(top, se);
+  if (!(f < ft)) return 0u;
+  const float steps = (TZ > 1 ? 0.15f : 0.04f) * static_cast<float>(nx + ny + nz);
+  return static_cast<unsigned>((ft - f) / ft * fminf(steps, 1.0e6f));
 }
 
-__global__ void adj_ring_init_kernel(unsigned long long *ring, unsigned long long slots) {
-  for (unsigned long long i = blockIdx.x * static_cast<unsigned long long>(blockDim.x) + threadIdx.x;
-       i < slots; i += static_cast<unsigned long long>(gridDim.x) * blockDim.x)
-    ring[i] = slot_free(i);
-}
-
-// Queue the tiles holding a cell that is ready from the start.
+// Queue the tiles holding a ready cell: reached, not done, and no neighbour that
+// is not done names its side.  blockIdx.y: problem (first + y).
 template <int TX, int TY, int TZ>
-__global__ void adj_tile_seed_kernel(const AdjProb *probs, int nprob, int64_t total, TileQueue q) {
-  for (int64_t g = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; g < total;
-       g += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const AdjProb &P = probs[find_adj_prob(probs, nprob, g)];
-    const int64_t n = g - P.base;
-    if (P.status[n] != 1 || P.cnt[n] != 0 || P.cnt_out[n] != 0) continue;
+__global__ void adj_tile_seed_kernel(const AdjProb *probs, int first, SolveParams sp) {
+  const AdjProb &P = probs[first + blockIdx.y];
+  const int64_t total = P.nx * P.ny * P.nz;
+  const unsigned char *const mask = P.mask;
+  const int64_t sy = P.nx, sz = P.nx * P.ny;
+  for (int64_t n = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; n < total;
+       n += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    if ((mask[n] & (kPending | kDone)) != kPending) continue;
     const Cell e = cell_of(P, n);
-    tq_activate(q, tile_of_cell<TX, TY, TZ>(P, e.c[0], e.c[1], e.c[2]));
+    // neighbour at n + d waits for n, its side `side`
+    auto uses = [&](int64_t d, int side) { return ((mask[n + d] >> side) & 1u) && !(mask[n + d] & kDone); };
+    const bool used = (e.c[0] > 0 && uses(-1, 1)) || (e.c[0] + 1 < P.nx && uses(1, 0)) ||
+                      (e.c[1] > 0 && uses(-sy, 3)) || (e.c[1] + 1 < P.ny && uses(sy, 2)) ||
+                      (P.ndim == 3 && ((e.c[2] > 0 && uses(-sz, 5)) || (e.c[2] + 1 < P.nz && uses(sz, 4))));
+    if (used) continue;
+    const unsigned tx = static_cast<unsigned>(e.c[0] / TX), ty = static_cast<unsigned>(e.c[1] / TY),
+                   tz = static_cast<unsigned>(e.c[2] / TZ);
+    activate(sp, static_cast<unsigned long long>(P.tile_base) + (tz * P.nty + ty) * P.ntx + tx, 0u,
+             tile_bucket<TX, TY, TZ>(P, tx, ty, tz));
   }
 }
 
-// Persistent CTAs, one thread per cell of a tile.  In this schedule a
-// processed cell m publishes the products p_k(m) = fl(lambda_m * W_k(m)) in
-// place of its weights W_k(m) (its upwind cells need nothing else from it) and
-// dL/ds; lambda itself is not stored.
-//
-// A visit takes a snapshot: a pending cell may be processed in this visit only
-// if its cross-tile count read 0 (acquire) when the visit started; the products
-// of its downwind neighbours across the tile edge are then final and are read
-// once.  The visit is a Kahn queue in shared memory with one block barrier per
-// round: the cells of the round's list, packed into the first threads so that
-// a round's FP64 work occupies as few warps as possible, sum g and the
-// products of their downwind neighbours in the fixed order (x-, x+, y-, y+,
-// z-, z+), form their own products, and release their upwind cells in the tile;
-// a cell whose in-tile count reaches zero joins the next round's list.  After
-// the last round each thread publishes its own cell if it was processed, the
-// tile is handed back, and the cross-tile releases follow (after a fence),
-// queueing a tile whose cell's count reaches zero.  A cross-tile count that
-// reaches zero during a visit marks the tile for another visit.
-#ifndef EIK_ADJ_TILE_MINB
-#define EIK_ADJ_TILE_MINB 4
-#endif
-// TIMING: per-CTA clocks of the visit phases and of the waits for work (the
-// eik_stats timing fields); without it those reads compile out.
+// TIMING: clocks of the visit phases and of the waits for work (the eik_stats
+// timing fields); without it those reads compile out.
 template <int D, int TX, int TY, int TZ, bool TIMING>
-__global__ void __launch_bounds__(TX * TY * TZ, (EIK_ADJ_TILE_MINB * 256 + TX * TY * TZ - 1) /
-                                                     (TX * TY * TZ)) adj_tiles_kernel(
-    const AdjProb *probs, int nprob, TileQueue q) {
-  constexpr int NT = TX * TY * TZ;
-  constexpr unsigned kClear = 0x40u, kDid = 0x80u;   // s_flags; bits 0..2D-1: halo sides
-  __shared__ double s_pw[D][NT];           // W_k, replaced by p_k once processed
-  __shared__ double s_halo[2 * D][NT];     // product of the neighbour across the tile edge
-  __shared__ double s_g[NT];
-  __shared__ double s_lam[NT];
-  __shared__ double s_coef[NT];
-  __shared__ int s_cnt[NT];
-  __shared__ unsigned char s_mask[NT];
-  __shared__ unsigned char s_flags[NT];
-  __shared__ unsigned short s_list[2][NT];
-  __shared__ int s_n[3];
-  __shared__ long long s_tile;
-  __shared__ int s_prob;
-  const int tid = threadIdx.x;
-  const unsigned lane = threadIdx.x & 31u;
-  const int lc[3] = {tid % TX, (tid / TX) % TY, tid / (TX * TY)};
-  constexpr int tdim[3] = {TX, TY, TZ};
-  constexpr int lstride[3] = {1, TX, TX * TY};
-  const unsigned long long reached = ld_rlx_u64(&q.ctl->reached);
+__global__ void __launch_bounds__(32, kAdjCtas) adj_tiles_kernel(const AdjProb *probs, int nprob, AdjCtl *ctl,
+                                                                SolveParams sp) {
+  using S = ATile<D, TX, TY, TZ>;
+  constexpr int NT = S::NT, NC = S::NC, HZ = S::HZ, SX = S::SX, SY = S::SY;
+  static_assert(NT % 32 == 0 && NT <= 256, "whole warps, 8-bit list entries");
+  constexpr int kStride[3] = {1, SX, SX * SY};
+  constexpr int kTile[3] = {TX, TY, TZ};
+  __shared__ S s;
+  const int lane = threadIdx.x;
+  auto pos_of = [](int q) { return ((q / (TX * TY) + HZ) * SY + (q / TX) % TY + 1) * SX + q % TX + 1; };
   unsigned long long visits = 0, rounds = 0, visit_ns = 0, idle_ns = 0, cyc[4] = {0, 0, 0, 0};
-  long long t_claim = 0, c0 = 0;
+  long long idle_since = 0, t_mark = 0, c0 = 0;
+  auto lap = [&](int i) {
+    if constexpr (TIMING) {
+      const long long c1 = clock64();
+      cyc[i] += static_cast<unsigned long long>(c1 - c0);
+      c0 = c1;
+    }
+  };
+  if constexpr (TIMING) {
+    c0 = clock64();
+    t_mark = now_ns();
+  }
 #pragma unroll 1
   for (;;) {
-    if (tid == 0) {
-      long long t_wait = 0;
-      if constexpr (TIMING) {
-        c0 = clock64();
-        t_wait = grid::now_ns();
-      }
-      long long tile = tq_pop(q, reached);
-      if constexpr (TIMING) {
-        t_claim = grid::now_ns();
-        idle_ns += static_cast<unsigned long long>(t_claim - t_wait);
-      }
-      int pi = 0;
-      if (tile >= 0) {
-        // queued -> being visited; activations from now on set bit 0 again
-        if (atomicExch(q.state + tile, kTRunning) != kTActive) {
-          tq_fail(q);                                 // a queued tile is claimed once
-          tile = -1;
-        } else {
-          __threadfence();                            // the claim before the tile's loads
-          pi = find_tile_prob(probs, nprob, tile);
-        }
-      }
-      s_tile = tile;
-      s_prob = pi;
-      s_n[0] = s_n[1] = s_n[2] = 0;
-      if constexpr (TIMING) {
-        const long long c1 = clock64();
-        cyc[0] += static_cast<unsigned long long>(c1 - c0);
-        c0 = c1;
-      }
-    }
-    __syncthreads();
-    const long long tile = s_tile;
-    if (tile < 0) break;
-    {
-    const AdjProb &P = probs[s_prob];
-    const int64_t lt = tile - P.tile_base;
-    const int64_t tx = lt % P.ntx, rest = lt / P.ntx;
-    const int64_t gc[3] = {tx * TX + lc[0], (rest % P.nty) * TY + lc[1], (rest / P.nty) * TZ + lc[2]};
-    const int64_t ext[3] = {P.nx, P.ny, P.nz};
-    const int64_t gstride[3] = {1, P.nx, P.nx * P.ny};
-    const bool present = gc[0] < P.nx && gc[1] < P.ny && gc[2] < P.nz;
-    const int64_t n = present ? (gc[2] * P.ny + gc[1]) * P.nx + gc[0] : 0;
-    // loads that do not depend on the cross-tile counts first, so that they are
-    // in flight together with the acquire below
-    unsigned st = 0u, mk = 0u, hm_out = 0u;
-    double g = 0.0, coef = 0.0, pw[D];
-    int cnt0 = 0;
-    if (present) {
-      st = ld_rlx_u8(P.status + n);
-      mk = P.mask[n];
-      cnt0 = ld_rlx_s32(P.cnt + n);
-      g = P.g ? P.g[n] : 0.0;
-      coef = P.grad[n];
-    }
-#pragma unroll
-    for (int k = 0; k < D; ++k) pw[k] = present ? ld_rlx_d(P.W[k] + n) : 0.0;
-#pragma unroll
-    for (int j = 0; j < 2 * D; ++j) {
-      const int k = j >> 1;
-      const bool up = j & 1;
-      const int l = lc[k] + (up ? 1 : -1);
-      const int64_t c = gc[k] + (up ? 1 : -1);
-      if (!present || (l >= 0 && l < tdim[k]) || c < 0 || c >= ext[k]) continue;
-      const int64_t m = n + (up ? gstride[k] : -gstride[k]);
-      if ((P.mask[m] >> (j ^ 1)) & 1u) hm_out |= 1u << j;   // this cell is m's side j^1
-    }
-    const bool pending = st == 1u;
-    const bool out_clear = pending && ld_acq_s32(P.cnt_out + n) == 0;
-    unsigned flags = out_clear ? kClear : 0u;
-#pragma unroll
-    for (int j = 0; j < 2 * D; ++j) {
-      if (!out_clear || !((hm_out >> j) & 1u)) continue;
-      const int k = j >> 1;
-      const int64_t m = n + ((j & 1) ? gstride[k] : -gstride[k]);
-      s_halo[j][tid] = ld_rlx_d(P.W[k] + m);                 // m's product, final
-      flags |= 1u << j;
-    }
-    s_g[tid] = g;
-    s_coef[tid] = coef;
-    s_cnt[tid] = pending ? cnt0 : -1;             // -1: no release ever targets it
-    s_mask[tid] = static_cast<unsigned char>(mk);
-    s_flags[tid] = static_cast<unsigned char>(flags);
-#pragma unroll
-    for (int k = 0; k < D; ++k) s_pw[k][tid] = pw[k];
-    if (out_clear && cnt0 == 0) s_list[0][atomicAdd(&s_n[0], 1)] = static_cast<unsigned short>(tid);
-    }
-    __syncthreads();
-    if (TIMING && tid == 0) {
-      const long long c1 = clock64();
-      cyc[1] += static_cast<unsigned long long>(c1 - c0);
-      c0 = c1;
-    }
-    unsigned long long processed = 0;
-    int round = 0;
+    long long tile = -1;
+    unsigned slot = 0, lo = 0;
 #pragma unroll 1
-    for (; round <= NT; ++round) {
-      // the entry is read together with the count (an unused slot holds some
-      // earlier cell index, masked into the tile)
-      const int n_cur = s_n[round % 3];
-      const int c_any = s_list[round & 1][tid] & (NT - 1);
-      if (n_cur == 0) break;
-      processed += static_cast<unsigned long long>(n_cur);
-      if (tid == 0) s_n[(round + 2) % 3] = 0;       // last read in the previous round
-      if ((tid & ~31) < n_cur) {                    // warp-uniform
-        const bool live = tid < n_cur;
-        const int c = live ? c_any : 0;
-        const int cc[3] = {c % TX, (c / TX) % TY, c / (TX * TY)};
-        // every shared load of the round first (addresses depend on c only), so
-        // that their latencies overlap; then the FP64 chain; then the releases
-        int nb[2 * D];
-        bool inb[2 * D];
-#pragma unroll
-        for (int j = 0; j < 2 * D; ++j) {
-          const int k = j >> 1;
-          const int l = cc[k] + ((j & 1) ? 1 : -1);
-          inb[j] = l >= 0 && l < tdim[k];
-          nb[j] = inb[j] ? c + ((j & 1) ? lstride[k] : -lstride[k]) : c;
-        }
-        const unsigned fc = s_flags[c];
-        const unsigned mc = s_mask[c];
-        double lam = s_g[c];
-        unsigned mn[2 * D], fu[2 * D];
-        double tv[2 * D], th[2 * D];
-#pragma unroll
-        for (int j = 0; j < 2 * D; ++j) {
-          mn[j] = s_mask[nb[j]];
-          fu[j] = s_flags[nb[j]];
-          tv[j] = s_pw[j >> 1][nb[j]];
-          th[j] = s_halo[j][c];                        // used only where flagged
-        }
-        unsigned fresh = 0u;                          // sides whose upwind cell became ready
-        if (live) {
-#pragma unroll
-          for (int j = 0; j < 2 * D; ++j) {
-            const bool halo = (fc >> j) & 1u;
-            if (halo || (inb[j] && ((mn[j] >> (j ^ 1)) & 1u))) lam = __dadd_rn(lam, halo ? th[j] : tv[j]);
-          }
-          s_lam[c] = lam;
-#pragma unroll
-          for (int k = 0; k < D; ++k)
-            if ((mc >> (2 * k)) & 3u) s_pw[k][c] = __dmul_rn(lam, s_pw[k][c]);
-          s_flags[c] = static_cast<unsigned char>(fc | kDid);
-          int old[2 * D];
-#pragma unroll
-          for (int j = 0; j < 2 * D; ++j)
-            old[j] = (((mc >> j) & 1u) && inb[j]) ? atomicSub(&s_cnt[nb[j]], 1) : 0;
-#pragma unroll
-          for (int j = 0; j < 2 * D; ++j)
-            if (old[j] == 1 && (fu[j] & kClear)) fresh |= 1u << j;
-        }
-        // append the cells made ready, one shared atomic per warp
-        unsigned total = 0u, below = 0u;
-        const unsigned lt_mask = (1u << lane) - 1u;
-#pragma unroll
-        for (int j = 0; j < 2 * D; ++j) {
-          const unsigned b = __ballot_sync(kFullMask, (fresh >> j) & 1u);
-          below += __popc(b & lt_mask);
-          total += __popc(b);
-        }
-        int base = 0;
-        if (n_cur <= 32) {                           // warp 0 alone appends this round
-          if (lane == 0) s_n[(round + 1) % 3] = static_cast<int>(total);
-        } else {
-          if (lane == 0 && total) base = atomicAdd(&s_n[(round + 1) % 3], static_cast<int>(total));
-          base = __shfl_sync(kFullMask, base, 0);
-        }
-        if (fresh) {
-          int pos = base + static_cast<int>(below);
-          // below counts the lower lanes' entries of every side; this lane's own
-          // entries take the next slots in side order
-          unsigned short *out = s_list[(round + 1) & 1];
-#pragma unroll
-          for (int j = 0; j < 2 * D; ++j)
-            if ((fresh >> j) & 1u) out[pos++] = static_cast<unsigned short>(nb[j]);
-        }
-      }
-      __syncthreads();
-    }
-    if (TIMING && tid == 0) {
-      const long long c1 = clock64();
-      cyc[2] += static_cast<unsigned long long>(c1 - c0);
-      c0 = c1;
-    }
-    // the cell of this thread again (not kept in registers over the rounds)
-    const AdjProb &P = probs[s_prob];
-    const int64_t lt = tile - P.tile_base;
-    const int64_t tx = lt % P.ntx, rest = lt / P.ntx;
-    const int64_t gc[3] = {tx * TX + lc[0], (rest % P.nty) * TY + lc[1], (rest / P.nty) * TZ + lc[2]};
-    const int64_t gstride[3] = {1, P.nx, P.nx * P.ny};
-    const bool present = gc[0] < P.nx && gc[1] < P.ny && gc[2] < P.nz;
-    const int64_t n = present ? (gc[2] * P.ny + gc[1]) * P.nx + gc[0] : 0;
-    const unsigned fl = s_flags[tid];
-    const unsigned mk = s_mask[tid];
-    const bool did = (fl & kDid) != 0u;
-    if (did) {
-      if (mk) P.grad[n] = __dmul_rn(s_lam[tid], s_coef[tid]);
-#pragma unroll
-      for (int k = 0; k < D; ++k)
-        if ((mk >> (2 * k)) & 3u) st_rlx_d(P.W[k] + n, s_pw[k][tid]);
-      P.status[n] = 2;
-    } else if (s_cnt[tid] >= 0) {
-      P.cnt[n] = s_cnt[tid];                               // the in-tile releases of this visit
-    }
-    __threadfence();                                       // results before hand-back and releases
-    __syncthreads();
-    if (tid == 0) {
-      if (processed) atomicAdd(&q.ctl->done, processed);
-      ++visits;
-      rounds += static_cast<unsigned long long>(round);
-      // end of the visit: back to idle, or queued again when activated meanwhile
-      if (atomicCAS(q.state + tile, kTRunning, 0u) != kTRunning) {
-        atomicExch(q.state + tile, kTActive);
-        tq_push(q, static_cast<unsigned>(tile));
+    for (;;) {
+      const unsigned long long e = pop_entry(sp, idle_since, slot, lo);
+      if (e == kEmpty) break;
+      int f = -1;
+      if (lane == 0) f = try_claim(sp, e & 0xffffffffull, static_cast<unsigned>(e >> 32));
+      f = __shfl_sync(kFull, f, 0);
+      if (f >= 0) { tile = static_cast<long long>(e & 0xffffffffull); break; }
+      if (lane == 0) {
+        atomicAdd(&sp.ctl->run[slot * kCounterPad], 0xffffffffu);
+        atomicAdd(&sp.ctl->work, -1);
       }
     }
-    if (did) {
+    if (tile < 0) break;
+    idle_since = 0;
+    ++visits;
+    if constexpr (TIMING) {
+      const long long now = now_ns();
+      idle_ns += static_cast<unsigned long long>(now - t_mark);
+      t_mark = now;
+    }
+    lap(0);
+    // the problem's record through the read-only path: the fence below would
+    // send each of these reads to L2
+    const AdjProb &P = probs[find_tile_prob(probs, nprob, static_cast<unsigned>(tile))];
+    const int64_t nx = ldg_i64(&P.nx), ny = ldg_i64(&P.ny), nz = ldg_i64(&P.nz);
+    unsigned tc[3];
+    {   // fewer than 2^31 tiles: 32-bit divisions
+      const unsigned lt = static_cast<unsigned>(tile - ldg_i64(&P.tile_base)),
+                     ntx = static_cast<unsigned>(ldg_i64(&P.ntx)), nty = static_cast<unsigned>(ldg_i64(&P.nty));
+      const unsigned rest = lt / ntx;
+      tc[0] = lt - rest * ntx;
+      tc[2] = rest / nty;
+      tc[1] = rest - tc[2] * nty;
+    }
+    const int64_t x0 = static_cast<int64_t>(tc[0]) * TX, y0 = static_cast<int64_t>(tc[1]) * TY,
+                  z0 = static_cast<int64_t>(tc[2]) * TZ;
+    const int64_t sy = nx, sz = nx * ny, first = z0 * sz + y0 * sy + x0;
+    unsigned char *const mask = reinterpret_cast<unsigned char *>(ldg_i64(&P.mask)) + first;
+    double *const grad = reinterpret_cast<double *>(ldg_i64(&P.grad)) + first;
+    const double *const gin = reinterpret_cast<const double *>(ldg_i64(&P.g));
+    double *W[D];
+#pragma unroll
+    for (int ax = 0; ax < D; ++ax) W[ax] = reinterpret_cast<double *>(ldg_i64(&P.W[ax])) + first;
+    fence_ar();      // the claim is ordered before the tile's loads
+    const int xlo = x0 > 0 ? -1 : 0, ylo = y0 > 0 ? -1 : 0, zlo = z0 > 0 ? -1 : 0;
+    const int xhi = nx - x0 > TX ? TX + 1 : static_cast<int>(nx - x0);
+    const int yhi = ny - y0 > TY ? TY + 1 : static_cast<int>(ny - y0);
+    const int zhi = nz - z0 > TZ ? TZ + 1 : static_cast<int>(nz - z0);
+    double coef[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      const int q = k * 32 + lane, ps = pos_of(q);
+      const int ix = q % TX, iy = (q / TX) % TY, iz = q / (TX * TY);
+      const bool in = ix < xhi && iy < yhi && iz < zhi;
+      const int64_t off = iz * sz + iy * sy + ix;
+      s.m[ps] = static_cast<unsigned char>(in ? ld_rlx_u8(mask + off) : 0u);
+      coef[k] = in ? grad[off] : 0.0;
+      s.lam[q] = in && gin ? gin[first + off] : 0.0;
+#pragma unroll
+      for (int ax = 0; ax < D; ++ax) s.p[ax][ps] = in ? ld_rlx_d(W[ax] + off) : 0.0;
+    }
+    constexpr int FX = TY * TZ, FY = TX * TZ, FZ = (D == 3) ? TX * TY : 0;
+    constexpr int H = 2 * FX + 2 * FY + 2 * FZ, HC = (H + 31) / 32;
+    // halo faces: y (x fastest: coalesced), z, x.  face j of halo cell i
+    auto halo = [](int i, int &ix, int &iy, int &iz) -> int {
+      if (i < 2 * FY) {
+        const int j = i % FY;
+        ix = j % TX; iz = j / TX; iy = i < FY ? -1 : TY;
+        return i < FY ? 2 : 3;
+      }
+      if (i < 2 * FY + 2 * FZ) {
+        const int k = i - 2 * FY, j = k % (FZ > 0 ? FZ : 1);
+        ix = j % TX; iy = j / TX; iz = k < FZ ? -1 : TZ;
+        return k < FZ ? 4 : 5;
+      }
+      const int k = i - 2 * FY - 2 * FZ, j = k % FX;
+      iy = j % TY; iz = j / TY; ix = k < FX ? -1 : TX;
+      return k < FX ? 0 : 1;
+    };
+    unsigned hm[HC];
+#pragma unroll
+    for (int c = 0; c < HC; ++c) {
+      const int i = c * 32 + lane;
+      int ix, iy, iz;
+      halo(i, ix, iy, iz);
+      const bool in = i < H && ix >= xlo && ix < xhi && iy >= ylo && iy < yhi && iz >= zlo && iz < zhi;
+      hm[c] = in ? ld_rlx_u8(mask + iz * sz + iy * sy + ix) : 0u;
+      if (i < H) s.m[((iz + HZ) * SY + iy + 1) * SX + ix + 1] = static_cast<unsigned char>(hm[c]);
+    }
+    fence_ar();      // a user seen done has its products published
+#pragma unroll
+    for (int c = 0; c < HC; ++c) {
+      const int i = c * 32 + lane;
+      int ix, iy, iz;
+      const int j = halo(i, ix, iy, iz);
+      if (i < H && (hm[c] & kDone) && ((hm[c] >> (j ^ 1)) & 1u))
+        s.p[j >> 1][((iz + HZ) * SY + iy + 1) * SX + ix + 1] =
+            ld_rlx_d(W[j >> 1] + iz * sz + iy * sy + ix);
+    }
+    __syncwarp();
+    // word k of these sets in lane k: cells to do, cells with a user across the
+    // tile edge that is not done, cells with a user in the tile across face j
+    unsigned todo_w = 0u, blocked_w = 0u, user_w[2 * D];
+#pragma unroll
+    for (int j = 0; j < 2 * D; ++j) user_w[j] = 0u;
+#pragma unroll 1
+    for (int k = 0; k < NC; ++k) {
+      const int q = k * 32 + lane, ps = pos_of(q);
+      const int cc[3] = {q % TX, (q / TX) % TY, q / (TX * TY)};
+      const unsigned own = s.m[ps];
+      bool blocked = false;
 #pragma unroll
       for (int j = 0; j < 2 * D; ++j) {
-        if (!((mk >> j) & 1u)) continue;
-        const int k = j >> 1;
-        const bool up = j & 1;
-        const int l = lc[k] + (up ? 1 : -1);
-        if (l >= 0 && l < tdim[k]) continue;
-        if (atomicSub(P.cnt_out + n + (up ? gstride[k] : -gstride[k]), 1) == 1) {
-          __threadfence();                                 // the release before the activation
-          int64_t uc[3] = {gc[0], gc[1], gc[2]};
-          uc[k] += up ? 1 : -1;
-          tq_activate(q, tile_of_cell<TX, TY, TZ>(P, uc[0], uc[1], uc[2]));
+        const int ax = j >> 1;
+        const unsigned mn = s.m[ps + ((j & 1) ? kStride[ax] : -kStride[ax])];
+        const bool user = (mn >> (j ^ 1)) & 1u, inside = cc[ax] != ((j & 1) ? kTile[ax] - 1 : 0);
+        blocked = blocked || (user && !inside && !(mn & kDone));
+        const unsigned b = __ballot_sync(kFull, user && inside);
+        if (lane == k) user_w[j] = b;
+      }
+      const unsigned bt = __ballot_sync(kFull, (own & kPending) && !(own & kDone));
+      const unsigned bb = __ballot_sync(kFull, blocked);
+      if (lane == k) { todo_w = bt; blocked_w = bb; }
+    }
+    const unsigned todo0_w = todo_w;
+    lap(1);
+#pragma unroll 1
+    for (int round = 0; round <= NT; ++round) {
+      unsigned ready_w = todo_w & ~blocked_w;
+#pragma unroll
+      for (int j = 0; j < 2 * D; ++j) ready_w &= ~(user_w[j] & face_bits<TX, TY, TZ>(todo_w, j));
+      const int n = list_of_set<NC>(ready_w, s.list);
+      __syncwarp();
+      if (n == 0) break;
+      ++rounds;
+      todo_w &= ~ready_w;
+#pragma unroll 1
+      for (int b = lane; b < n; b += 32) {
+        const int q = s.list[b], ps = pos_of(q);
+        double lam = s.lam[q];
+        const unsigned own = s.m[ps];
+#pragma unroll
+        for (int j = 0; j < 2 * D; ++j) {
+          const int nb = ps + ((j & 1) ? kStride[j >> 1] : -kStride[j >> 1]);
+          const unsigned mn = s.m[nb];
+          const double pr = s.p[j >> 1][nb];
+          if ((mn >> (j ^ 1)) & 1u) lam = __dadd_rn(lam, pr);
+        }
+#pragma unroll
+        for (int ax = 0; ax < D; ++ax)
+          if ((own >> (2 * ax)) & 3u) s.p[ax][ps] = __dmul_rn(lam, s.p[ax][ps]);
+        s.lam[q] = lam;
+      }
+      __syncwarp();
+    }
+    lap(2);
+    const unsigned done_w = todo0_w & ~todo_w;
+    if (__any_sync(kFull, done_w != 0u)) {
+      const bool whole = !__any_sync(kFull, todo_w != 0u);   // no later visit reads this tile's products
+      unsigned out_any = 0u, ndone = 0u;
+#pragma unroll
+      for (int k = 0; k < NC; ++k) {
+        const unsigned w = __shfl_sync(kFull, done_w, k);
+        ndone += __popc(w);
+        if (!((w >> lane) & 1u)) continue;
+        const int q = k * 32 + lane, ps = pos_of(q);
+        const int cc[3] = {q % TX, (q / TX) % TY, q / (TX * TY)};
+        const int64_t off = cc[2] * sz + cc[1] * sy + cc[0];
+        const unsigned own = s.m[ps];
+        if (own & 0x3fu) grad[off] = __dmul_rn(s.lam[q], coef[k]);
+#pragma unroll
+        for (int ax = 0; ax < D; ++ax) {
+          const bool out_lo = ((own >> (2 * ax)) & 1u) && cc[ax] == 0;
+          const bool out_hi = ((own >> (2 * ax + 1)) & 1u) && cc[ax] == kTile[ax] - 1;
+          if (out_lo) out_any |= 1u << (2 * ax);
+          if (out_hi) out_any |= 1u << (2 * ax + 1);
+          if (out_lo || out_hi || (!whole && ((own >> (2 * ax)) & 3u))) st_rlx_d(W[ax] + off, s.p[ax][ps]);
         }
       }
+      fence_ar();                               // products before the mask bytes that name them done
+#pragma unroll
+      for (int k = 0; k < NC; ++k) {
+        const unsigned w = __shfl_sync(kFull, done_w, k);
+        if (!((w >> lane) & 1u)) continue;
+        const int q = k * 32 + lane;
+        const int64_t off = (q / (TX * TY)) * sz + ((q / TX) % TY) * sy + q % TX;
+        mask[off] = static_cast<unsigned char>(s.m[pos_of(q)] | kDone);
+      }
+      out_any = __reduce_or_sync(kFull, out_any);
+      fence_ar();                               // the mask bytes before the activations
+      __syncwarp();
+      if ((out_any >> lane) & 1u) {                  // an upwind cell on face j lies in the grid
+        const int ax = lane >> 1, d = (lane & 1) ? 1 : -1;
+        const unsigned ux = tc[0] + (ax == 0 ? d : 0), uy = tc[1] + (ax == 1 ? d : 0), uz = tc[2] + (ax == 2 ? d : 0);
+        activate(sp, static_cast<unsigned long long>(P.tile_base) + (uz * P.nty + uy) * P.ntx + ux, 0u,
+                 tile_bucket<TX, TY, TZ>(P, ux, uy, uz), lo);
+      }
+      __syncwarp();
+      if (lane == 0) atomicAdd(&ctl->done, static_cast<unsigned long long>(ndone));
     }
-    if (TIMING && tid == 0) {
-      visit_ns += static_cast<unsigned long long>(grid::now_ns() - t_claim);
-      cyc[3] += static_cast<unsigned long long>(clock64() - c0);
+    if (lane == 0) {
+      finish_tile(sp, static_cast<unsigned long long>(tile));
+      fence_ar();
+      atomicAdd(&sp.ctl->run[slot * kCounterPad], 0xffffffffu);
+      atomicAdd(&sp.ctl->work, -1);
+    }
+    __syncwarp();
+    lap(3);
+    if constexpr (TIMING) {
+      const long long now = now_ns();
+      visit_ns += static_cast<unsigned long long>(now - t_mark);
+      t_mark = now;
     }
   }
-  if (tid == 0) {
-    atomicAdd(&q.ctl->visits, visits);
-    atomicAdd(&q.ctl->rounds, rounds);
-    atomicAdd(&q.ctl->ctas, 1ull);
+  if (lane == 0) {
+    atomicAdd(&ctl->visits, visits);
+    atomicAdd(&ctl->rounds, rounds);
+    atomicAdd(&ctl->ctas, 1ull);
     if constexpr (TIMING) {
-      atomicAdd(&q.ctl->visit_ns, visit_ns);
-      atomicAdd(&q.ctl->idle_ns, idle_ns);
+      atomicAdd(&ctl->visit_ns, visit_ns);
+      atomicAdd(&ctl->idle_ns, idle_ns);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) atomicAdd(&q.ctl->cycles[i], cyc[i]);
+      for (int i = 0; i < 4; ++i) atomicAdd(&ctl->cycles[i], cyc[i]);
     }
   }
 }
@@ -757,7 +726,7 @@ cudaError_t launch_adjoint(const AdjProb *probs_dev, int nprob, int64_t total, A
   int64_t g = (total + 255) / 256;
   if (g > 8 * sms()) g = 8 * sms();
   if (g < 1) g = 1;
-  adj_setup_kernel<<<static_cast<int>(g), 256, 0, stream>>>(probs_dev, nprob, total, ctl, 0, 0, 0);
+  adj_setup_kernel<<<static_cast<int>(g), 256, 0, stream>>>(probs_dev, nprob, total, ctl);
   adj_seed_kernel<<<static_cast<int>(g), 256, 0, stream>>>(probs_dev, nprob, total, ctl, front);
   note_launches(2);
   cudaError_t e = cudaGetLastError();
@@ -786,59 +755,53 @@ cudaError_t launch_adjoint(const AdjProb *probs_dev, int nprob, int64_t total, A
 namespace {
 
 template <int D, int TX, int TY, int TZ>
-cudaError_t run_tiles(const AdjProb *probs_dev, int nprob, int64_t total, int64_t total_tiles,
-                      TileQueue q, unsigned long long qcap, int ctas_per_sm, bool timing,
-                      cudaStream_t stream) {
-  int64_t g = (total + 255) / 256;
-  if (g > 8 * sms()) g = 8 * sms();
-  if (g < 1) g = 1;
-  int64_t gr = (static_cast<int64_t>(qcap) + 255) / 256;
-  if (gr > 8 * sms()) gr = 8 * sms();
-  adj_ring_init_kernel<<<static_cast<int>(gr), 256, 0, stream>>>(q.ring, qcap);
-  adj_setup_kernel<<<static_cast<int>(g), 256, 0, stream>>>(probs_dev, nprob, total, q.ctl, TX, TY, TZ);
-  adj_tile_seed_kernel<TX, TY, TZ><<<static_cast<int>(g), 256, 0, stream>>>(probs_dev, nprob, total, q);
-  note_launches(3);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  // persistent CTAs, all resident (a cooperative launch guarantees it): an idle
-  // CTA waits for tiles that running CTAs queue
-  constexpr int NT = TX * TY * TZ;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, adj_tiles_kernel<D, TX, TY, TZ, true>, NT, 0);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
+cudaError_t run_tiles(const AdjProb *probs_dev, int nprob, int64_t total, int64_t total_tiles, AdjCtl *ctl,
+                      const SolveParams &sp, int ctas_per_sm, bool timing, bool resume, cudaStream_t stream) {
+  int64_t gx = (total / nprob + 255) / 256, share = (static_cast<int64_t>(sms()) * 8 + nprob - 1) / nprob;
+  if (gx > share) gx = share;
+  if (gx < 1) gx = 1;
+  for (int first = 0; first < nprob && !resume; first += 65535) {
+    const unsigned n = static_cast<unsigned>(nprob - first < 65535 ? nprob - first : 65535);
+    adj_setup_tiles_kernel<<<dim3(static_cast<unsigned>(gx), n), 256, 0, stream>>>(probs_dev, first, ctl);
+    note_launches(1);
+  }
+  for (int first = 0; first < nprob; first += 65535) {
+    const unsigned n = static_cast<unsigned>(nprob - first < 65535 ? nprob - first : 65535);
+    adj_tile_seed_kernel<TX, TY, TZ><<<dim3(static_cast<unsigned>(gx), n), 256, 0, stream>>>(probs_dev, first, sp);
+    note_launches(1);
+  }
+  int per_sm = kAdjCtas;
   if (ctas_per_sm > 0 && per_sm > ctas_per_sm) per_sm = ctas_per_sm;
   int64_t blocks = static_cast<int64_t>(sms()) * per_sm;
   if (blocks > total_tiles) blocks = total_tiles;
   if (blocks < 1) blocks = 1;
-  void *args[] = {const_cast<AdjProb **>(&probs_dev), &nprob, &q};
-  const void *fn = timing ? reinterpret_cast<const void *>(adj_tiles_kernel<D, TX, TY, TZ, true>)
-                          : reinterpret_cast<const void *>(adj_tiles_kernel<D, TX, TY, TZ, false>);
-  e = cudaLaunchCooperativeKernel(fn, dim3(static_cast<unsigned>(blocks)), dim3(NT), args, 0, stream);
+  if (timing)
+    adj_tiles_kernel<D, TX, TY, TZ, true><<<static_cast<int>(blocks), 32, 0, stream>>>(probs_dev, nprob, ctl, sp);
+  else
+    adj_tiles_kernel<D, TX, TY, TZ, false><<<static_cast<int>(blocks), 32, 0, stream>>>(probs_dev, nprob, ctl, sp);
   note_launches(1);
-  return e;
+  return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_adjoint_tiles(const AdjProb *probs_dev, int nprob, int64_t total,
-                                 int64_t total_tiles, int ndim, AdjCtl *ctl, unsigned *tile_state,
-                                 unsigned long long *queue, unsigned long long qcap,
-                                 int ctas_per_sm, long long timeout_ns, bool timing,
-                                 cudaStream_t stream) {
-  if (total_tiles < 1 || qcap < static_cast<unsigned long long>(total_tiles) || (qcap & (qcap - 1)))
-    return cudaErrorInvalidValue;
-  TileQueue q;
-  q.state = tile_state;
-  q.ring = queue;
-  q.mask = qcap - 1ull;
-  q.ctl = ctl;
-  q.timeout_ns = timeout_ns;
+cudaError_t launch_adj_h2s(const double *v, int v_is_slowness, double hh, int64_t n, double *hs,
+                           cudaStream_t stream) {
+  int64_t g = (n + 255) / 256;
+  if (g > 8 * sms()) g = 8 * sms();
+  adj_h2s_kernel<<<static_cast<int>(g < 1 ? 1 : g), 256, 0, stream>>>(v, v_is_slowness, hh, n, hs);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_adjoint_tiles(const AdjProb *probs_dev, int nprob, int64_t total, int64_t total_tiles,
+                                 int ndim, AdjCtl *ctl, const SolveParams &sp, int ctas_per_sm, bool timing,
+                                 bool resume, cudaStream_t stream) {
   if (ndim == 3)
-    return run_tiles<3, kAdjTile3[0], kAdjTile3[1], kAdjTile3[2]>(probs_dev, nprob, total, total_tiles,
-                                                                  q, qcap, ctas_per_sm, timing, stream);
-  return run_tiles<2, kAdjTile2[0], kAdjTile2[1], kAdjTile2[2]>(probs_dev, nprob, total, total_tiles,
-                                                                q, qcap, ctas_per_sm, timing, stream);
+    return run_tiles<3, kAdjTile3[0], kAdjTile3[1], kAdjTile3[2]>(probs_dev, nprob, total, total_tiles, ctl, sp,
+                                                                  ctas_per_sm, timing, resume, stream);
+  return run_tiles<2, kAdjTile2[0], kAdjTile2[1], kAdjTile2[2]>(probs_dev, nprob, total, total_tiles, ctl, sp,
+                                                                ctas_per_sm, timing, resume, stream);
 }
 
 }  // namespace eik

@@ -6,7 +6,9 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <mutex>
+#include <tuple>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -131,25 +133,30 @@ Workspace &ws() { return g_ws_dev[g_dev]; }
 
 struct AdjWorkspace {
   int device = -1;
-  DevBuf<int> cnt, cnt_out;
-  DevBuf<double> W, lam;
-  DevBuf<unsigned char> mask, status;
-  DevBuf<unsigned long long> front, ring;
-  DevBuf<unsigned> tile_state;
+  DevBuf<int> cnt;
+  DevBuf<double> W, lam, hs;
+  DevBuf<unsigned char> mask;
+  DevBuf<unsigned long long> front, tmax;
+  // the tile schedule's scheduler
+  DevBuf<unsigned long long> state, slots;
+  DevBuf<Ctl> sched;
   DevBuf<eik::AdjProb> probs;
   DevBuf<eik::AdjCtl> ctl;
   DevBuf<int64_t> src;
   DevBuf<double> gsum;                   // per-problem gradients summed into shared outputs
   DevBuf<const double *> gptr;           // their addresses, grouped by output
   eik::AdjCtl *ctl_host = nullptr;
+  unsigned *sched_host = nullptr;        // pinned: the scheduler's status
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
 
   void release_all() {
-    cnt.release(); cnt_out.release(); W.release(); lam.release(); mask.release();
-    status.release(); front.release(); ring.release(); tile_state.release();
+    cnt.release(); W.release(); lam.release(); hs.release(); mask.release(); front.release(); tmax.release();
+    state.release(); slots.release(); sched.release();
     probs.release(); ctl.release(); src.release(); gsum.release(); gptr.release();
     if (ctl_host) cudaFreeHost(ctl_host);
     ctl_host = nullptr;
+    if (sched_host) cudaFreeHost(sched_host);
+    sched_host = nullptr;
     if (ev0) cudaEventDestroy(ev0);
     if (ev1) cudaEventDestroy(ev1);
     ev0 = ev1 = nullptr;
@@ -1803,20 +1810,25 @@ extern "C" eik_status eik_adjoint(const eik_problem *probs, int nprob, const dou
     total_tiles += ntile[(size_t)i * 3] * ntile[(size_t)i * 3 + 1] * ntile[(size_t)i * 3 + 2];
   }
   if (tiles && total_tiles >= (int64_t(1) << 31)) { set_err("adjoint: too many tiles"); return EIK_EINVAL; }
-  const uint64_t qcap = next_pow2((uint64_t)std::max<int64_t>(total_tiles, 2));
   if (!adj().ctl_host) CK(cudaMallocHost(&adj().ctl_host, sizeof(eik::AdjCtl)), "adjoint: pinned");
-  CK(adj().cnt.ensure((size_t)total), "adjoint: alloc counts");
+  // frontier ring: every tile has at most one live entry, so a slot holds few
+  // more than total_tiles; a quarter of that at first (a full slot: the run goes
+  // on with more room)
+  const uint64_t full_cap = next_pow2((uint64_t)std::max<int64_t>(total_tiles, 16));
+  uint64_t cap = std::min(full_cap, next_pow2((uint64_t)total_tiles / 4 + 1024));
+  const int naxes = same_ndim ? hps[0].ndim : 3;
   if (tiles) {
-    CK(adj().cnt_out.ensure((size_t)total), "adjoint: alloc counts");
-    CK(adj().status.ensure((size_t)total), "adjoint: alloc status");
-    CK(adj().tile_state.ensure((size_t)total_tiles), "adjoint: alloc tile states");
-    CK(adj().ring.ensure((size_t)qcap), "adjoint: alloc tile queue");
+    CK(adj().state.ensure((size_t)total_tiles), "adjoint: alloc tile states");
+    CK(adj().sched.ensure(1), "adjoint: alloc scheduler");
+    CK(adj().tmax.ensure((size_t)nprob), "adjoint: alloc largest times");
+    if (!adj().sched_host) CK(cudaMallocHost(&adj().sched_host, sizeof(unsigned)), "adjoint: pinned");
   } else {
+    CK(adj().cnt.ensure((size_t)total), "adjoint: alloc counts");
     CK(adj().front.ensure((size_t)total * 2), "adjoint: alloc frontiers");
+    CK(adj().lam.ensure((size_t)total), "adjoint: alloc lambda");
   }
-  CK(adj().W.ensure((size_t)total * 3), "adjoint: alloc weights");
+  CK(adj().W.ensure((size_t)total * naxes), "adjoint: alloc weights");
   CK(adj().mask.ensure((size_t)total), "adjoint: alloc masks");
-  if (!tiles) CK(adj().lam.ensure((size_t)total), "adjoint: alloc lambda");
   CK(adj().probs.ensure((size_t)nprob), "adjoint: alloc problems");
   CK(adj().ctl.ensure(1), "adjoint: alloc control");
   CK(adj().src.ensure((size_t)std::max<int64_t>(total_src, 1)), "adjoint: alloc sources");
@@ -1842,14 +1854,29 @@ extern "C" eik_status eik_adjoint(const eik_problem *probs, int nprob, const dou
     CK(adj().gsum.ensure((size_t)total), "adjoint: alloc summed gradients");
     CK(adj().gptr.ensure((size_t)nprob), "adjoint: alloc gradient table");
   }
+  // models that several problems share: fl(h^2 s) once per cell
+  std::vector<int> model_of((size_t)nprob);            // first problem with the same model
+  std::vector<int> uses((size_t)nprob, 0);
+  std::map<std::tuple<const double *, double, int64_t>, int> models;
+  std::vector<int64_t> hs_off((size_t)nprob, -1);
+  int64_t hs_cells = 0;
+  for (int i = 0; i < nprob; ++i) {
+    const HostProblem &hp = hps[(size_t)i];
+    const int m = models.emplace(std::make_tuple(hp.speed, hp.h, hp.n), i).first->second;
+    model_of[(size_t)i] = m;
+    if (++uses[(size_t)m] == 2) {
+      hs_off[(size_t)m] = hs_cells;
+      hs_cells += hps[(size_t)m].n;
+    }
+  }
+  if (hs_cells) CK(adj().hs.ensure((size_t)hs_cells), "adjoint: alloc shared models");
   std::vector<eik::AdjProb> ap((size_t)nprob);
   std::vector<int64_t> all_src;
   int64_t base = 0, tile_base = 0;
   for (int i = 0; i < nprob; ++i) {
     const HostProblem &hp = hps[(size_t)i];
     eik::AdjProb &A = ap[(size_t)i];
-    A.cnt_out = tiles ? adj().cnt_out.p + base : nullptr;
-    A.status = tiles ? adj().status.p + base : nullptr;
+    A.tmax = tiles ? adj().tmax.p + i : nullptr;
     A.ntx = ntile[(size_t)i * 3];
     A.nty = ntile[(size_t)i * 3 + 1];
     A.ntz = ntile[(size_t)i * 3 + 2];
@@ -1858,12 +1885,15 @@ extern "C" eik_status eik_adjoint(const eik_problem *probs, int nprob, const dou
     A.t = hp.out;
     A.v = hp.speed;
     A.v_is_slowness = from_slowness(opts);
+    const int64_t ho = hs_off[(size_t)model_of[(size_t)i]];
+    A.hs = ho >= 0 ? adj().hs.p + ho : nullptr;
     A.g = dL_dt ? dL_dt[i] : nullptr;
     A.grad = sum_shared ? adj().gsum.p + base : dL_dslowness[i];
     A.lam = tiles ? nullptr : adj().lam.p + base;
-    for (int k = 0; k < 3; ++k) A.W[k] = adj().W.p + (size_t)k * (size_t)total + base;
+    for (int k = 0; k < 3; ++k)
+      A.W[k] = k < naxes ? adj().W.p + (size_t)k * (size_t)total + base : nullptr;
     A.mask = adj().mask.p + base;
-    A.cnt = adj().cnt.p + base;
+    A.cnt = tiles ? nullptr : adj().cnt.p + base;
     A.src_idx = adj().src.p + all_src.size();
     A.nsrc = (int64_t)hp.src.size();
     A.nx = hp.dims[2];
@@ -1880,46 +1910,73 @@ extern "C" eik_status eik_adjoint(const eik_problem *probs, int nprob, const dou
                        cudaMemcpyHostToDevice, s), "adjoint: upload sources");
   CK(cudaMemcpyAsync(adj().probs.p, ap.data(), ap.size() * sizeof(eik::AdjProb),
                      cudaMemcpyHostToDevice, s), "adjoint: upload problems");
-  CK(cudaMemsetAsync(adj().cnt.p, 0, (size_t)total * sizeof(int), s), "adjoint: clear counts");
-  if (tiles) {
-    CK(cudaMemsetAsync(adj().cnt_out.p, 0, (size_t)total * sizeof(int), s), "adjoint: clear counts");
-    CK(cudaMemsetAsync(adj().tile_state.p, 0, (size_t)total_tiles * sizeof(unsigned), s),
-       "adjoint: clear tile states");
-  }
-  CK(cudaMemsetAsync(adj().ctl.p, 0, sizeof(eik::AdjCtl), s), "adjoint: clear control");
   const int64_t tmo_ms = opts && opts->timeout_ms > 0 ? opts->timeout_ms : 60000;
   if (!adj().ev0) {
     CK(cudaEventCreate(&adj().ev0), "adjoint: event");
     CK(cudaEventCreate(&adj().ev1), "adjoint: event");
   }
   CK(cudaEventRecord(adj().ev0, s), "adjoint: event record");
-  if (tiles)
-    CK(eik::launch_adjoint_tiles(adj().probs.p, nprob, total, total_tiles, hps[0].ndim, adj().ctl.p,
-                                 adj().tile_state.p, adj().ring.p, qcap,
-                                 opts ? opts->ctas_per_sm : 0, tmo_ms * 1000000ll,
-                                 opts && opts->counters, s),
-       "adjoint launch");
-  else
-    CK(eik::launch_adjoint(adj().probs.p, nprob, total, adj().ctl.p, adj().front.p,
-                           tmo_ms * 1000000ll, s), "adjoint launch");
-  if (sum_shared) {
-    std::vector<const double *> table;
-    std::vector<size_t> first;
-    for (size_t g = 0; g < group_out.size(); ++g) {
-      first.push_back(table.size());
-      for (int i : group_of[g]) table.push_back(ap[(size_t)i].grad);
-    }
-    CK(cudaMemcpyAsync(adj().gptr.p, table.data(), table.size() * sizeof(const double *),
-                       cudaMemcpyHostToDevice, s), "adjoint: upload gradient table");
-    for (size_t g = 0; g < group_out.size(); ++g) {
-      CK(eik::launch_sum_ordered(adj().gptr.p + first[g], (int)group_of[g].size(), group_out[g],
-                                 hps[(size_t)group_of[g][0]].n, s), "adjoint: ordered sum");
-    }
+  for (int i = 0; i < nprob; ++i) {
+    if (hs_off[(size_t)i] >= 0)
+      CK(eik::launch_adj_h2s(hps[(size_t)i].speed, from_slowness(opts), hps[(size_t)i].h * hps[(size_t)i].h,
+                             hps[(size_t)i].n, adj().hs.p + hs_off[(size_t)i], s), "adjoint: shared model");
   }
-  CK(cudaEventRecord(adj().ev1, s), "adjoint: event record");
-  CK(cudaMemcpyAsync(adj().ctl_host, adj().ctl.p, sizeof(eik::AdjCtl), cudaMemcpyDeviceToHost, s),
-     "adjoint: read status");
-  CK(cudaStreamSynchronize(s), "adjoint");
+  unsigned sched_status = 0;
+  for (bool resume = false;; resume = true) {
+    if (tiles) {
+      CK(adj().slots.ensure((size_t)(cap * eik::kNumSlots)), "adjoint: alloc frontier");
+      if (!resume) {
+        CK(cudaMemsetAsync(adj().ctl.p, 0, sizeof(eik::AdjCtl), s), "adjoint: clear control");
+        CK(cudaMemsetAsync(adj().tmax.p, 0, (size_t)nprob * sizeof(unsigned long long), s),
+           "adjoint: clear largest times");
+      }
+      CK(cudaMemsetAsync(adj().sched.p, 0, sizeof(Ctl), s), "adjoint: clear scheduler");
+      CK(cudaMemsetAsync(adj().state.p, 0, (size_t)total_tiles * sizeof(unsigned long long), s),
+         "adjoint: clear tile states");
+      CK(cudaMemsetAsync(adj().slots.p, 0, (size_t)(cap * eik::kNumSlots) * sizeof(unsigned long long), s),
+         "adjoint: clear frontier");
+      SolveParams sp;
+      std::memset(&sp, 0, sizeof(sp));
+      sp.state = adj().state.p;
+      sp.slots = adj().slots.p;
+      sp.cap_mask = (unsigned)(cap - 1);
+      sp.ctl = adj().sched.p;
+      sp.timeout_ns = tmo_ms * 1000000ll;
+      sp.window = 31;
+      CK(eik::launch_adjoint_tiles(adj().probs.p, nprob, total, total_tiles, hps[0].ndim, adj().ctl.p, sp,
+                                   opts ? opts->ctas_per_sm : 0, opts && opts->counters, resume, s),
+         "adjoint launch");
+      CK(cudaMemcpyAsync(adj().sched_host, &adj().sched.p->status, sizeof(unsigned), cudaMemcpyDeviceToHost, s),
+         "adjoint: read scheduler status");
+    } else {
+      CK(cudaMemsetAsync(adj().cnt.p, 0, (size_t)total * sizeof(int), s), "adjoint: clear counts");
+      CK(cudaMemsetAsync(adj().ctl.p, 0, sizeof(eik::AdjCtl), s), "adjoint: clear control");
+      CK(eik::launch_adjoint(adj().probs.p, nprob, total, adj().ctl.p, adj().front.p,
+                             tmo_ms * 1000000ll, s), "adjoint launch");
+    }
+    if (sum_shared) {
+      std::vector<const double *> table;
+      std::vector<size_t> first;
+      for (size_t g = 0; g < group_out.size(); ++g) {
+        first.push_back(table.size());
+        for (int i : group_of[g]) table.push_back(ap[(size_t)i].grad);
+      }
+      CK(cudaMemcpyAsync(adj().gptr.p, table.data(), table.size() * sizeof(const double *),
+                         cudaMemcpyHostToDevice, s), "adjoint: upload gradient table");
+      for (size_t g = 0; g < group_out.size(); ++g) {
+        CK(eik::launch_sum_ordered(adj().gptr.p + first[g], (int)group_of[g].size(), group_out[g],
+                                   hps[(size_t)group_of[g][0]].n, s), "adjoint: ordered sum");
+      }
+    }
+    CK(cudaEventRecord(adj().ev1, s), "adjoint: event record");
+    CK(cudaMemcpyAsync(adj().ctl_host, adj().ctl.p, sizeof(eik::AdjCtl), cudaMemcpyDeviceToHost, s),
+       "adjoint: read status");
+    CK(cudaStreamSynchronize(s), "adjoint");
+    sched_status = tiles ? *adj().sched_host : 0u;
+    // a bucket slot overflowed: go on with more room
+    if (sched_status != eik::kEcapacity || cap >= 4 * full_cap || cap >= (1u << 29)) break;
+    cap *= 4;
+  }
   const eik::AdjCtl &c = *adj().ctl_host;
   if (stats) {
     std::memset(stats, 0, sizeof(*stats));
@@ -1934,8 +1991,12 @@ extern "C" eik_status eik_adjoint(const eik_problem *probs, int nprob, const dou
     float ms = 0.f;
     if (cudaEventElapsedTime(&ms, adj().ev0, adj().ev1) == cudaSuccess) stats->solve_ms = ms;
   }
-  if (c.status == eik::kEtimeout) { set_err("adjoint: device wait timed out"); return EIK_ETIMEOUT; }
-  if (c.status != 0) return EIK_ECUDA;
+  if (c.status == eik::kEtimeout || sched_status == eik::kEtimeout) {
+    set_err("adjoint: device wait timed out");
+    return EIK_ETIMEOUT;
+  }
+  if (sched_status == eik::kEcapacity) { set_err("adjoint: frontier capacity exhausted"); return EIK_ECAPACITY; }
+  if (c.status != 0 || sched_status != 0) return EIK_ECUDA;
   if (c.done != c.reached) { set_err("adjoint: %llu of %llu cells processed",
                                      (unsigned long long)c.done, (unsigned long long)c.reached);
                              return EIK_ECUDA; }

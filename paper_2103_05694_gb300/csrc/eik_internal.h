@@ -277,16 +277,16 @@ struct AdjProb {
   const double *t;          // forward arrival times (the exact fixed point)
   const double *v;          // speed (slowness s when v_is_slowness: v = fl(1/s))
   int v_is_slowness;
+  const double *hs;         // fl(h^2 s) per cell where problems share v (else NULL)
   const double *g;          // dL/dt (NULL: 0)
   double *grad;             // dL/ds output
   double *lam;              // adjoint variable (workspace; NULL in the tile schedule)
   double *W[3];             // per axis: weight of the axis' upwind side(s) (workspace); in
                             // the tile schedule lambda * weight once the cell is processed
-  unsigned char *mask;      // upwind sides (bit 2k + side) of each cell (workspace)
-  int *cnt;                 // downwind users not yet processed (workspace); with tiles:
-                            // the users inside the cell's own tile
-  int *cnt_out;             // with tiles: the users in other tiles (workspace)
-  unsigned char *status;    // with tiles: 0 unreached, 1 pending, 2 processed (workspace)
+  unsigned char *mask;      // upwind sides (bit 2k + side) of each cell (workspace); with
+                            // tiles bit 6: reached, bit 7: processed
+  int *cnt;                 // levels: downwind users not yet processed (workspace)
+  unsigned long long *tmax; // tiles: the largest time, rounded down to its high word (workspace)
   const int64_t *src_idx;   // sorted unique sources
   int64_t nsrc;
   int64_t nx, ny, nz;
@@ -299,7 +299,7 @@ struct AdjProb {
 
 // Control block of the adjoint.  Level-synchronous schedule: frontier counts
 // rotate over three slots: level L reads slot L % 3, appends to (L + 1) % 3 and
-// clears (L + 2) % 3.  Tile schedule: queue counters and visit statistics.
+// clears (L + 2) % 3.  Tile schedule: visit statistics.
 struct AdjCtl {
   unsigned long long reached;        // cells with a finite time
   unsigned long long pad0[15];
@@ -313,10 +313,6 @@ struct AdjCtl {
   unsigned long long levels;
   unsigned status;
   unsigned pad4[13];
-  unsigned long long head;           // tile schedule: queue tickets taken and pushed
-  unsigned long long pad5[15];
-  unsigned long long tail;
-  unsigned long long pad6[15];
   unsigned long long visits;         // tile visits
   unsigned long long rounds;         // rounds summed over tile visits
   unsigned long long visit_ns;       // visit time summed over CTAs
@@ -331,28 +327,21 @@ struct AdjCtl {
 // entries.
 cudaError_t launch_adjoint(const AdjProb *probs_dev, int nprob, int64_t total, AdjCtl *ctl,
                            unsigned long long *front, long long timeout_ns, cudaStream_t stream);
-// The tile schedule: set-up with counts split by tile, the initial queue, and a
-// persistent launch that relaxes ready tiles in shared memory.  tile_state
-// holds total_tiles words, zero on entry; queue holds qcap slots (a power of two
-// >= total_tiles, set up by the launch).  ndim: of every problem (one tile shape
-// per launch).  The tiles are kAdjTile2 in 2D and kAdjTile3 in 3D.  ctas_per_sm
-// caps the persistent CTAs per SM (0: occupancy).
-// 2D adjoint tile (compile-time): 16x8 cells, 8 resident CTAs of 128 threads per SM
-// (32-source tomography adjoint 11.6 ms, against 12.9 ms with 16x16 tiles at 4
-// CTAs per SM, 14.0 with 32x8 and 15.7 with 32x16)
-#ifndef EIK_ADJ_TILE2_X
-#define EIK_ADJ_TILE2_X 16
-#endif
-#ifndef EIK_ADJ_TILE2_Y
-#define EIK_ADJ_TILE2_Y 8
-#endif
-constexpr int kAdjTile2[3] = {EIK_ADJ_TILE2_X, EIK_ADJ_TILE2_Y, 1};
-constexpr int kAdjTile3[3] = {8, 8, 4};
-// timing: collect the visit and wait clocks (eik_stats timing fields).
-cudaError_t launch_adjoint_tiles(const AdjProb *probs_dev, int nprob, int64_t total,
-                                 int64_t total_tiles, int ndim, AdjCtl *ctl, unsigned *tile_state,
-                                 unsigned long long *queue, unsigned long long qcap,
-                                 int ctas_per_sm, long long timeout_ns, bool timing,
-                                 cudaStream_t stream);
+// hs[i] = fl(hh fl(1 / v[i])) (v_is_slowness: of the speed fl(1 / v[i])).
+cudaError_t launch_adj_h2s(const double *v, int v_is_slowness, double hh, int64_t n, double *hs,
+                           cudaStream_t stream);
+// The tile schedule: set-up, the initial queue, and a persistent launch of one
+// warp per tile on the bucket scheduler of sp (state, slots and ctl zero on
+// entry; every tile has at most one live entry).  ndim: of
+// every problem (one tile shape per launch).  ctas_per_sm caps the persistent
+// CTAs per SM (0: kAdjCtas).  timing: collect the visit and wait clocks.
+// resume: go on where a launch ended for a full bucket slot (visits always
+// commit): no set-up, the tiles with ready cells are queued anew.
+constexpr int kAdjTile2[3] = {16, 16, 1};
+constexpr int kAdjTile3[3] = {8, 4, 4};
+constexpr int kAdjCtas = 12;
+cudaError_t launch_adjoint_tiles(const AdjProb *probs_dev, int nprob, int64_t total, int64_t total_tiles,
+                                 int ndim, AdjCtl *ctl, const SolveParams &sp, int ctas_per_sm, bool timing,
+                                 bool resume, cudaStream_t stream);
 
 }  // namespace eik
