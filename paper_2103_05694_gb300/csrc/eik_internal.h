@@ -210,8 +210,11 @@ struct SeedItem {
   double t0;
 };
 
+// t_min: no item is earlier (the scheduler starts at its bucket).  lower: the
+// items only lower values of a field that is kept (see seed_kernel).
 cudaError_t launch_seed(const SolveParams &p, const SeedItem *items, int64_t nitems,
-                        double k_delta, double delta_fixed, cudaStream_t stream);
+                        double k_delta, double delta_fixed, cudaStream_t stream, double t_min = 0.0,
+                        bool lower = false);
 cudaError_t launch_reseed(const SolveParams &p, const Prob *host_probs, int nprob,
                           cudaStream_t stream);
 cudaError_t launch_persistent(const SolveParams &p, int grid, cudaStream_t stream);

@@ -707,14 +707,19 @@ __device__ __forceinline__ unsigned long long tile_of(const Prob &P, int64_t x, 
 }
 
 // Boundary nodes: t := t0 and activate, with every cell to be evaluated, the
-// tile of the source and the tiles of its in-grid neighbours.
+// tile of the source and the tiles of its in-grid neighbours.  The scheduler's
+// hint starts at t_min's bucket: from 0, items beyond the ring's reach would all
+// be clamped to its last slot, in no order.  lower: t := min(t, t0), and nothing
+// is activated where t stays (the node is fixed at a value the field agrees with).
 __global__ void seed_kernel(SolveParams p, const SeedItem *__restrict__ items, int64_t n,
-                            double k_delta, double delta_fixed, int tx_, int ty_, int tz_) {
+                            double k_delta, double delta_fixed, int tx_, int ty_, int tz_,
+                            double t_min, bool lower) {
   Ctl *ctl = p.ctl;
   double delta = delta_fixed > 0.0 ? delta_fixed
                                    : k_delta * (ctl->rsum / static_cast<double>(ctl->rcount));
   if (!(delta > 0.0) || !(bits_of(delta) < kInfBits)) delta = 1.0;
   const double inv = 1.0 / delta;
+  const unsigned base = bucket_of_time(bits_of(t_min), static_cast<float>(inv));
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl->delta = delta;
     ctl->inv_delta = inv;
@@ -726,13 +731,15 @@ __global__ void seed_kernel(SolveParams p, const SeedItem *__restrict__ items, i
        i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const SeedItem it = items[i];
     const Prob &P = p.probs[it.prob];
-    P.t[it.idx] = it.t0;
+    const bool stays = lower && !(it.t0 < P.t[it.idx]);
+    if (!stays) P.t[it.idx] = it.t0;
     const int64_t x = it.idx % P.nx, yz = it.idx / P.nx;
     const int64_t y = yz % P.ny, z = yz / P.ny;
     const unsigned long long own = tile_of(P, x, y, z, tx_, ty_, tz_);
     p.tile_src[own] = 1;
+    if (stays) continue;
     const unsigned b = bucket_of_time(bits_of(it.t0), static_cast<float>(inv));
-    activate(p, own, 1u << kFaceFull, b);
+    activate(p, own, 1u << kFaceFull, b, base);
     const int64_t c3[3] = {x, y, z};
     const int64_t n3[3] = {P.nx, P.ny, P.nz};
     for (int k = 0; k < 3; ++k) {
@@ -741,7 +748,7 @@ __global__ void seed_kernel(SolveParams p, const SeedItem *__restrict__ items, i
         q[k] += side ? 1 : -1;
         if (q[k] < 0 || q[k] >= n3[k]) continue;
         const unsigned long long nt = tile_of(P, q[0], q[1], q[2], tx_, ty_, tz_);
-        if (nt != own) activate(p, nt, 1u << kFaceFull, b);
+        if (nt != own) activate(p, nt, 1u << kFaceFull, b, base);
       }
     }
   }
@@ -972,11 +979,16 @@ static void tile_dims(const SolveParams &p, int &tx, int &ty, int &tz) {
 }
 
 cudaError_t launch_seed(const SolveParams &p, const SeedItem *items, int64_t nitems,
-                        double k_delta, double delta_fixed, cudaStream_t stream) {
+                        double k_delta, double delta_fixed, cudaStream_t stream, double t_min,
+                        bool lower) {
+  if (t_min > 0.0) {   // the pushes below lower the hint to the smallest bucket
+    const cudaError_t e = cudaMemsetAsync(&p.ctl->cur, 0xff, sizeof(p.ctl->cur), stream);
+    if (e != cudaSuccess) return e;
+  }
   int tx, ty, tz;
   tile_dims(p, tx, ty, tz);
   const int grid = grid_for(nitems > 0 ? nitems : 1, 4);
-  seed_kernel<<<grid, 256, 0, stream>>>(p, items, nitems, k_delta, delta_fixed, tx, ty, tz);
+  seed_kernel<<<grid, 256, 0, stream>>>(p, items, nitems, k_delta, delta_fixed, tx, ty, tz, t_min, lower);
   note_launches(1);
   return cudaGetLastError();
 }
