@@ -72,9 +72,10 @@ typedef enum {
  * them for a given batch.
  * A solve whose scheduling options (delta, k_delta, window, band, ctas_per_sm, tile,
  * arith, sched_flags bits 0-2 and 5) are all zero, without counters, trace or
- * test_stall, runs the guided kernel, with its own tiles and buckets (one warp per
- * tile: 8x8 in 2D, 4x4x4 to 8x8x4 in 3D); capacity is then a lower bound.  Otherwise
- * the defaults below fill in the options that are zero.  They depend on how many
+ * test_stall, runs the front kernel (8x8 tiles in 2D, 4x4x4 in 3D, a thread per cell)
+ * or, in 3D with 8 or more sources and 40 million cells or more, the guided kernel (8x8x4
+ * tiles, one warp each), with their own buckets; capacity is then a lower bound.
+ * Otherwise the defaults below fill in the options that are zero.  They depend on how many
  * independent wavefronts the batch has:
  *   2D, fewer than 8 sources in the batch: 16x16 tiles, k_delta 16, window 16,
  *     band 16, 1 CTA per SM (latency-bound: one front);
@@ -109,7 +110,7 @@ typedef struct {
                               / sqrt(ndim), i.e. one cell's travel time; <= 0: default */
     int arith;             /* arithmetic of d-bar: 1 = FP64 unit, 2 = exact emulation on the
                               integer pipes (same results bit for bit); 0: default;
-                              3 = the guided kernel, whatever the other scheduling options
+                              3 = the front or guided kernel, whatever the other scheduling options
                               (counters, a trace, test_stall, update 1-3 or sched_flags bits
                               0-2 and 5 still select the other kernel, as with 0) */
     int sched_flags;       /* bit 0: the look-ahead window follows the lowest bucket holding

@@ -16,7 +16,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "_libeik.so")
-SOURCES = ["eik_solver.cu", "eik_guided.cu", "eik_api.cu", "eik_selftest.cu", "eik_noalloc.cu", "eik_adjoint.cu",
+SOURCES = ["eik_solver.cu", "eik_guided.cu", "eik_front.cu", "eik_api.cu", "eik_selftest.cu", "eik_noalloc.cu", "eik_adjoint.cu",
            "eik_ablation.cu", "eik_schedules.cu"]
 HEADERS = ["eik_internal.h", "eik_sched.cuh", "eik_exact.cuh", "eik_forms.cuh", "eik_grid.cuh",
            os.path.join("..", "..", "include", "eik.h")]

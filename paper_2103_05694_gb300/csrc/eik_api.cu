@@ -57,7 +57,7 @@ constexpr double kKDelta3[2] = {0.75, 0.375};   // single front, many fronts
 constexpr int kSingleFrontCtas3Small = 14;      // 3D tiles of at most 64 cells
 constexpr int kManyFronts = 8;                  // sources at which a solve counts as many fronts
 constexpr int kMaxRetries = 4;
-constexpr int kArithGuided = 3;                 // eik_opts.arith: the guided kernel
+constexpr int kArithGuided = 3;                 // eik_opts.arith: the front or guided kernel
 // eik_opts.sched_flags bits of the tomography interface
 constexpr int kFlagSlowness = 1 << 6;     // speed arrays hold slowness s; v = fl(1/s) is used
 constexpr int kFlagSumShared = 1 << 7;    // eik_adjoint: equal outputs receive the ordered sum
@@ -393,24 +393,32 @@ bool use_guided(const eik_opts *o) {
   return o->arith == 0 && o->tile == 0 && o->ctas_per_sm <= 0 && o->window <= 0 && !(o->band > 0) &&
          !(o->delta > 0) && !(o->k_delta > 0);
 }
-// Shape, bucket width, look-ahead and CTAs per SM of a guided solve.  A few
-// fronts are bound by the latency of the visits along them: small tiles.  With
-// many fronts, or one in a large volume, larger tiles cost fewer instructions
-// per cell (88-problem 3D batch: 8x8x4 70 ms, 8x4x4 88 ms, 4x4x4 113 ms; 256^3
-// checkerboard: 8x4x4 12.7 ms, 4x4x4 14.6 ms; one 97 x 131 x 203 grid: 4x4x4
-// 3.7 ms, 8x4x4 4.3 ms; 2D: 8x8 in all cases, 16x8 and 16x16 lost).
+// Kernel (by its shape), bucket width, look-ahead and CTAs per SM of a solve with
+// automatic options.  The front kernel wherever the length of the fronts bounds the
+// solve; with many fronts in a large volume there is ordered work for every warp,
+// and the guided kernel's fewer evaluations win (batches of 128^3 grids, front
+// against guided: 16.8 M cells 5.7 and 8.7 ms, 33.5 M 10.5 and 11.3, 67 M 20.8 and
+// 16.5, 185 M 58 and 36).  CTAs per SM: a single 2D front has few active tiles, and
+// more CTAs take tiles out of order (751 x 2301 section: 4 CTAs 4.1 ms, 8 4.9 ms,
+// 2 4.4 ms; 1502 x 4602: 9.4 ms, with 3 10.4 ms); elsewhere as many as fit (24
+// sections: 8 to 12 CTAs 1.9 ms, 16 2.3 ms; 256^3 checkerboard: 8 10.9 ms, 12 8.7,
+// 14 8.0, 20 with spills 9.3; 97 x 131 x 203: 12 1.76, 14 1.82, 16 2.1; many 3D
+// fronts launch the 20 of the other kernels, of which 14 run at a time).  Bucket
+// widths: the layered section 4.4 ms at 8, 4.2 at 16, 4.1 at 32; 32 sources of
+// 1024^2 11.0 ms at 2, 11.2 at 4, 11.6 at 16; 3D 1.80 ms (97 x 131 x 203) and 8.6 ms
+// (checkerboard) at 0.4, 1.74 and 9.0 at 0.75, 1.75 and 9.7 at 1.5.
 struct GuidedCfg {
-  int shape;        // of the guided shapes
+  int shape;
   double k_delta;
   int window;
-  int per_sm;       // CTAs (warps) per SM
+  int per_sm;
 };
 GuidedCfg guided_config(int ndim, int64_t total_sources, int64_t cells) {
   const bool many = total_sources >= kManyFronts;
-  if (ndim == 2) return many ? GuidedCfg{0, 4.0, 16, eik::kGuidedCtas} : GuidedCfg{0, 16.0, 16, 4};
-  const bool large = cells >= (int64_t(1) << 23);
-  if (many) return GuidedCfg{large ? 2 : 0, 0.75, 31, eik::kGuidedCtas};
-  return GuidedCfg{large ? 1 : 0, 0.75, 31, kSingleFrontCtas3Small};
+  if (ndim == 2)
+    return many ? GuidedCfg{eik::kFrontShape, 4.0, 16, eik::kFrontCtas2} : GuidedCfg{eik::kFrontShape, 32.0, 16, 4};
+  if (many && cells >= int64_t(40) * 1000 * 1000) return GuidedCfg{eik::kGuidedShape0, 0.75, 31, eik::kGuidedCtas};
+  return GuidedCfg{eik::kFrontShape, 0.5, 31, many ? eik::kGuidedCtas : eik::kFrontCtas3};
 }
 
 // Tile shape of opts (validated): shape index and cells per axis.  opts.tile 0
@@ -424,7 +432,7 @@ eik_status tile_shape(const eik_opts *opts, int ndim, int64_t total_sources, int
     return EIK_EINVAL;
   }
   if (use_guided(opts))
-    shape = eik::kGuidedShape0 + guided_config(ndim, total_sources, cells).shape;
+    shape = guided_config(ndim, total_sources, cells).shape;
   else
     shape = t == 0 ? auto_config(ndim, total_sources, int_arith).shape : t - 1;
   if (shape != 0 && int_arith) {

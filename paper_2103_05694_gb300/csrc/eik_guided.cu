@@ -1,4 +1,5 @@
-// Guided tile kernel: the default of lean solves with automatic options.
+// Guided tile kernel: lean solves with automatic options of 3D batches large
+// enough to fill the device with ordered work (the others: eik_front.cu).
 //
 // The asynchronous tile schedule of eik_solver.cu (same buckets, claims and
 // activations) with another way to relax a claimed tile.  That kernel finds
@@ -26,15 +27,12 @@
 // is deferred inside a visit: the look-ahead window only limits which tiles are
 // taken.
 //
-// What bounds it: with many fronts, instructions (88-problem 3D batch: issue 52 %
-// at 4.75 warps per scheduler, the instruction cache close to its request rate,
-// so loops are rolled and the scheduler's functions are not inlined: 218 -> 75 ms
-// for the 128-source 3D batch); with one front, the latency of the visits along it
-// (about 1300 cycles per round of exact evaluations).  Evaluations per cell: 2.5
-// (batch) and 4 (checkerboard) against 6.1 and 11.2 in the other kernel.
-// Measured against that kernel with the same d-bar (us): 129^2 grid 796 -> 613,
-// layered section 12286 -> 9417, 256^3 checkerboard 17345 -> 12597, 88-problem
-// batch 115674 -> 61437.
+// What bounds it: instructions (88-problem 3D batch: issue 52 % at 4.75 warps per
+// scheduler, the instruction cache close to its request rate, so loops are rolled
+// and the scheduler's functions are not inlined: 218 -> 75 ms for the 128-source
+// batch).  Evaluations per cell: 2.5 against 6.1 in the kernel of eik_solver.cu.
+// Measured against that kernel with the same d-bar: 88-problem batch 115.7 -> 57.4
+// ms.  Tiles: 8x8x4 70 ms, 8x4x4 88 ms, 4x4x4 113 ms (an earlier state).
 // Tried and dropped: a visit limit inside the tile (narrow windows leave partial
 // tiles: batch 75 -> 139 ms at a quarter of the bucket width); waiting while a
 // neighbour tile is being visited (visits halve, the wait costs more); skipping
@@ -69,46 +67,30 @@ __device__ __forceinline__ float offset_f(unsigned long long v, unsigned long lo
 }
 
 // First-order update in FP32 from the axis minima (offsets; +inf allowed), r = h / v.
-template <int D>
-__device__ __forceinline__ float root_f(const float (&a)[D], float r) {
-  float lo = fminf(a[0], a[1]), hi = fmaxf(a[0], a[1]), top = 0.0f;
-  if (D == 3) {
-    top = fmaxf(hi, a[D - 1]);
-    const float m = fminf(hi, a[D - 1]);
-    hi = fmaxf(lo, m);
-    lo = fminf(lo, m);
-  }
+__device__ __forceinline__ float root_f(const float (&a)[3], float r) {
+  float lo = fminf(a[0], a[1]), hi = fmaxf(a[0], a[1]);
+  const float top = fmaxf(hi, a[2]), m = fminf(hi, a[2]);
+  hi = fmaxf(lo, m);
+  lo = fminf(lo, m);
   float u = r;
   const float b1 = hi - lo;               // NaN when both are +inf: one-sided
   if (b1 < r) {
     const float rr = r * r;
     u = 0.5f * (b1 + ffa::sqrt_est(fmaf(-b1, b1, 2.0f * rr)));
-    if (D == 3) {
-      const float b2 = top - lo;
-      if (b2 < u) {
-        const float s = b1 + b2, q = fmaf(b1, b1, b2 * b2);
-        const float disc = fmaxf(fmaf(s, s, -3.0f * (q - rr)), 1e-30f);
-        u = (s + ffa::sqrt_est(disc)) * (1.0f / 3.0f);
-      }
+    const float b2 = top - lo;
+    if (b2 < u) {
+      const float s = b1 + b2, q = fmaf(b1, b1, b2 * b2);
+      const float disc = fmaxf(fmaf(s, s, -3.0f * (q - rr)), 1e-30f);
+      u = (s + ffa::sqrt_est(disc)) * (1.0f / 3.0f);
     }
   }
   return lo + u;
 }
 
-__device__ __forceinline__ int find_prob_ro(const SolveParams &p, unsigned tile) {
-  int lo = 0, hi = p.nprob - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (ldg_i64(&p.probs[mid].tile_base) <= static_cast<int64_t>(tile)) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
-template <int D, int TX, int TY, int TZ>
+template <int TX, int TY, int TZ>
 struct GTile {
   static constexpr int NT = TX * TY * TZ, NC = NT / 32;
-  static constexpr int HZ = D == 3 ? 1 : 0;
-  static constexpr int SX = TX + 2, SY = TY + 2, SZ = TZ + 2 * HZ, NS = SX * SY * SZ;
+  static constexpr int SX = TX + 2, SY = TY + 2, SZ = TZ + 2, NS = SX * SY * SZ;
   double t[NS];                    // exact values with halo
   unsigned long long c[NT];
   float g[NS];                     // predicted offsets with halo
@@ -117,10 +99,10 @@ struct GTile {
   unsigned char fell[NT];          // 1: fell since the last look
 };
 
-template <int D, int TX, int TY, int TZ>
+template <int TX, int TY, int TZ>
 __global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) {
-  using S = GTile<D, TX, TY, TZ>;
-  constexpr int NT = S::NT, NC = S::NC, HZ = S::HZ, SX = S::SX, SY = S::SY;
+  using S = GTile<TX, TY, TZ>;
+  constexpr int D = 3, NT = S::NT, NC = S::NC, SX = S::SX, SY = S::SY;
   static_assert(NT % 32 == 0 && NT <= 256, "whole warps, 8-bit list entries");
   constexpr int kStride[3] = {1, SX, SX * SY};
   constexpr int kTile[3] = {TX, TY, TZ};
@@ -129,7 +111,7 @@ __global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) 
   const float inv_delta = static_cast<float>(p.ctl->inv_delta);
   const int se = p.ctl->scale_exp;
   long long idle_since = 0;
-  auto pos_of = [](int q) { return ((q / (TX * TY) + HZ) * SY + (q / TX) % TY + 1) * SX + q % TX + 1; };
+  auto pos_of = [](int q) { return ((q / (TX * TY) + 1) * SY + (q / TX) % TY + 1) * SX + q % TX + 1; };
   auto nbrs = [](unsigned w, int j) { return face_bits<TX, TY, TZ>(w, j); };
 
 #pragma unroll 1
@@ -210,7 +192,7 @@ __global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) 
 #pragma unroll 1
     for (;;) {
       {  // halo faces: y (x fastest: coalesced), z, x
-        constexpr int FX = TY * TZ, FY = TX * TZ, FZ = (D == 3) ? TX * TY : 0;
+        constexpr int FX = TY * TZ, FY = TX * TZ, FZ = TX * TY;
         constexpr int H = 2 * FX + 2 * FY + 2 * FZ;
 #pragma unroll 4
         for (int i = lane; i < H; i += 32) {
@@ -219,14 +201,14 @@ __global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) 
             const int j = i % FY;
             ix = j % TX; iz = j / TX; iy = i < FY ? -1 : TY;
           } else if (i < 2 * FY + 2 * FZ) {
-            const int k = i - 2 * FY, j = k % (FZ > 0 ? FZ : 1);
+            const int k = i - 2 * FY, j = k % FZ;
             ix = j % TX; iy = j / TX; iz = k < FZ ? -1 : TZ;
           } else {
             const int k = i - 2 * FY - 2 * FZ, j = k % FX;
             iy = j % TY; iz = j / TY; ix = k < FX ? -1 : TX;
           }
           const bool in = ix >= xlo && ix < xhi && iy >= ylo && iy < yhi && iz >= zlo && iz < zhi;
-          s.t[((iz + HZ) * SY + iy + 1) * SX + ix + 1] =
+          s.t[((iz + 1) * SY + iy + 1) * SX + ix + 1] =
               in ? ld_time(T0 + iz * sz + iy * sy + ix) : from_bits(kInfBits);
         }
       }
@@ -268,7 +250,7 @@ __global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) 
         // 1. order: relax in FP32 by rows of 32 cells, up and down by turns, each row
         // while one of its neighbour rows (or itself) has fallen since its last turn
         unsigned stale = (1u << NC) - 1u;
-        constexpr int kReach = (TX * TY > 32 ? TX * TY : 32) / 32;   // rows hold neighbours up to +-kReach
+        static_assert(TX * TY == 64, "a slice is two rows");
 #pragma unroll 1
         for (int it = 0; stale && it < 4 * NT; ++it) {
 #pragma unroll 1
@@ -280,15 +262,13 @@ __global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) 
 #pragma unroll
             for (int ax = 0; ax < D; ++ax) a[ax] = fminf(s.g[ps - kStride[ax]], s.g[ps + kStride[ax]]);
             const float r = s.r[q];
-            const float nv = root_f<D>(a, r);
+            const float nv = root_f(a, r);
             const bool fell = !((fixed >> k) & 1u) && nv < s.g[ps] - kSettled * r;
             if (fell) s.g[ps] = nv;
             stale &= ~(1u << k);
             if (__any_sync(kFull, fell)) {
-              // rows k, k +- 1, and in 3D tiles of two rows per slice k +- 2
-              unsigned near = (7u << k) >> 1;
-              if (D == 3 && kReach == 2) near |= (17u << k) >> 2;
-              stale |= near & ((1u << NC) - 1u);
+              // rows k, k +- 1 and, in the next slices, k +- 2
+              stale |= (((7u << k) >> 1) | ((17u << k) >> 2)) & ((1u << NC) - 1u);
             }
             __syncwarp();
           }
@@ -465,22 +445,12 @@ __global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) 
   }
 }
 
-template <int D, int TX, int TY, int TZ>
-cudaError_t run_guided(const SolveParams &p, int grid, cudaStream_t stream) {
-  guided_kernel<D, TX, TY, TZ><<<grid, 32, 0, stream>>>(p);
-  return cudaGetLastError();
-}
-
 }  // namespace
 
 cudaError_t launch_guided(const SolveParams &p, int grid, cudaStream_t stream) {
   note_launches(1);
-  if (p.ndim == 2) return run_guided<2, 8, 8, 1>(p, grid, stream);
-  switch (p.tile_shape - kGuidedShape0) {
-    case 0: return run_guided<3, 4, 4, 4>(p, grid, stream);
-    case 1: return run_guided<3, 8, 4, 4>(p, grid, stream);
-    default: return run_guided<3, 8, 8, 4>(p, grid, stream);
-  }
+  guided_kernel<8, 8, 4><<<grid, 32, 0, stream>>>(p);
+  return cudaGetLastError();
 }
 
 }  // namespace eik

@@ -150,16 +150,15 @@ constexpr int resident_ctas(int tile_cells) {
 struct TileShape {
   int tx, ty, tz;
 };
-// The guided kernel's own shapes (one warp per tile) and the CTAs of one warp
-// per SM that its registers are bounded for.
-constexpr int kGuidedShape0 = kNumTileShapes;
+// The shapes of the kernels that choose them (eik_guided.cu and eik_front.cu), and
+// the CTAs per SM that their registers are bounded for.
+constexpr int kGuidedShape0 = kNumTileShapes;       // 8x8x4, one warp per tile
+constexpr int kFrontShape = kNumTileShapes + 1;     // 8x8, 4x4x4, a thread per cell
 constexpr int kGuidedCtas = 20;
+constexpr int kFrontCtas2 = 12, kFrontCtas3 = 14;
 __host__ __device__ inline TileShape tile_shape_of(int ndim, int shape) {
-  if (shape >= kGuidedShape0) {
-    const int g = shape - kGuidedShape0;
-    if (ndim == 3) return g == 0 ? TileShape{4, 4, 4} : g == 1 ? TileShape{8, 4, 4} : TileShape{8, 8, 4};
-    return TileShape{8, 8, 1};
-  }
+  if (shape == kGuidedShape0) return TileShape{8, 8, 4};
+  if (shape == kFrontShape) return ndim == 3 ? TileShape{4, 4, 4} : TileShape{8, 8, 1};
   if (ndim == 3) {
     switch (shape) {
       case 1: return TileShape{16, 4, 4};
@@ -218,8 +217,9 @@ cudaError_t launch_seed(const SolveParams &p, const SeedItem *items, int64_t nit
 cudaError_t launch_reseed(const SolveParams &p, const Prob *host_probs, int nprob,
                           cudaStream_t stream);
 cudaError_t launch_persistent(const SolveParams &p, int grid, cudaStream_t stream);
-// The guided kernel on its own tile shapes (tile_shape >= kGuidedShape0).
+// The guided and the front kernel (tile_shape kGuidedShape0 and kFrontShape).
 cudaError_t launch_guided(const SolveParams &p, int grid, cudaStream_t stream);
+cudaError_t launch_front(const SolveParams &p, int grid, cudaStream_t stream);
 cudaError_t launch_count_finite(const Prob *host_probs, int nprob, unsigned long long *out,
                                 cudaStream_t stream);
 // Finite times over every problem of a batch in one launch (adds into *out).

@@ -399,6 +399,15 @@ __device__ __forceinline__ int64_t ldg_i64(const void *p) {
   return __ldg(static_cast<const long long *>(p));
 }
 
+__device__ __forceinline__ int find_prob_ro(const SolveParams &p, unsigned tile) {
+  int lo = 0, hi = p.nprob - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (ldg_i64(&p.probs[mid].tile_base) <= static_cast<int64_t>(tile)) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
 constexpr float kInfF = __builtin_huge_valf();
 
 // A non-negative double (bit pattern) times 2^-se as a float, truncated; +inf stays.
@@ -447,33 +456,22 @@ __device__ __forceinline__ unsigned face_bits(unsigned w, int j) {
 }
 
 // A set's cells as a list in shared memory (to be read after a __syncwarp);
-// returns their number.  Every lane picks its bit of each word (few words: the
-// shorter chain, 210 against 435 cycles for 2), or each word's lane writes its
-// bits (many: fewer instructions, 14.7 against 29.0 kcycles a visit for 8).
+// returns their number.  Each word's lane writes its bits (every lane picking its
+// bit of each word in turn: 29.0 against 14.7 kcycles a visit for 8 words).
 template <int NC>
 __device__ __forceinline__ int list_of_set(unsigned set, unsigned char *list) {
   const int lane = threadIdx.x & 31;
-  int n = 0;
-  if constexpr (NC <= 2) {
+  const int own = __popc(set);
+  int n = own;
 #pragma unroll
-    for (int k = 0; k < NC; ++k) {
-      const unsigned w = __shfl_sync(kFull, set, k);
-      if ((w >> lane) & 1u) list[n + __popc(w & ((1u << lane) - 1u))] = static_cast<unsigned char>(k * 32 + lane);
-      n += __popc(w);
-    }
-  } else {
-    const int own = __popc(set);
-    n = own;
-#pragma unroll
-    for (int o = 1; o < NC; o <<= 1) {
-      const int v = __shfl_up_sync(kFull, n, o);
-      if (lane >= o) n += v;
-    }
-    int at = n - own;
-    n = __shfl_sync(kFull, n, NC - 1);
-#pragma unroll 1
-    for (unsigned w = set; w; w &= w - 1u) list[at++] = static_cast<unsigned char>(lane * 32 + __ffs(w) - 1);
+  for (int o = 1; o < NC; o <<= 1) {
+    const int v = __shfl_up_sync(kFull, n, o);
+    if (lane >= o) n += v;
   }
+  int at = n - own;
+  n = __shfl_sync(kFull, n, NC - 1);
+#pragma unroll 1
+  for (unsigned w = set; w; w &= w - 1u) list[at++] = static_cast<unsigned char>(lane * 32 + __ffs(w) - 1);
   return n;
 }
 

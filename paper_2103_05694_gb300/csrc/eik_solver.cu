@@ -1092,7 +1092,7 @@ int persistent_wide_blocks_per_sm(int ndim, int arith, int tile_shape) {
 }
 
 cudaError_t launch_persistent(const SolveParams &p, int grid, cudaStream_t stream) {
-  if (p.guided) return launch_guided(p, grid, stream);
+  if (p.guided) return p.tile_shape == kFrontShape ? launch_front(p, grid, stream) : launch_guided(p, grid, stream);
   cudaError_t e = cudaSuccess;
   EIK_SHAPE_SWITCH(p.ndim, p.tile_shape, e = S::launch(p, grid, stream));
   note_launches(1);
