@@ -31,6 +31,7 @@
 //    follow the cells it releases does not pay on this graph: in 2D most cells
 //    have two downwind users, so chains merge after about two steps while the
 //    few long chains stretch every frontier.)
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -770,8 +771,19 @@ cudaError_t run_tiles(const AdjProb *probs_dev, int nprob, int64_t total, int64_
     adj_tile_seed_kernel<TX, TY, TZ><<<dim3(static_cast<unsigned>(gx), n), 256, 0, stream>>>(probs_dev, first, sp);
     note_launches(1);
   }
-  int per_sm = kAdjCtas;
-  if (ctas_per_sm > 0 && per_sm > ctas_per_sm) per_sm = ctas_per_sm;
+  // ctas_per_sm 0: what the fronts can use (a front of a problem of n tiles is
+  // about n^(1/2) tiles in 2D, n^(2/3) in 3D), since idle warps only hold up the
+  // scheduler: 2D 9 problems of 700 x 700 with 2, 4, 8 and 12 per SM 3.28, 3.09, 3.27
+  // and 3.66 ms, 4 of 600 x 500 2.05, 2.08, 2.25 and 2.49 ms; 3D one of 100^3 2.65,
+  // 2.72, 3.25 and 4.06 ms, 4 of 110 x 90 x 100 4.88, 3.30, 3.01 and 3.33 ms
+  int per_sm = D == 3 ? 10 : kAdjCtas;
+  if (ctas_per_sm > 0) {
+    per_sm = ctas_per_sm < kAdjCtas ? ctas_per_sm : kAdjCtas;
+  } else {
+    const double each = static_cast<double>(total_tiles) / nprob;
+    const double want = nprob * (D == 3 ? 0.75 * cbrt(each) * cbrt(each) : 1.5 * sqrt(each)) / sms();
+    if (want < per_sm) per_sm = want > 2.0 ? static_cast<int>(ceil(want)) : 2;
+  }
   int64_t blocks = static_cast<int64_t>(sms()) * per_sm;
   if (blocks > total_tiles) blocks = total_tiles;
   if (blocks < 1) blocks = 1;

@@ -337,7 +337,7 @@ cudaError_t launch_adj_h2s(const double *v, int v_is_slowness, double hh, int64_
 // warp per tile on the bucket scheduler of sp (state, slots and ctl zero on
 // entry; every tile has at most one live entry).  ndim: of
 // every problem (one tile shape per launch).  ctas_per_sm caps the persistent
-// CTAs per SM (0: kAdjCtas).  timing: collect the visit and wait clocks.
+// CTAs per SM (0: chosen by the size).  timing: collect the visit and wait clocks.
 // resume: go on where a launch ended for a full bucket slot (visits always
 // commit): no set-up, the tiles with ready cells are queued anew.
 constexpr int kAdjTile2[3] = {16, 16, 1};
