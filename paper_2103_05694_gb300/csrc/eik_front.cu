@@ -171,6 +171,7 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
       if (lane == 0) fl->hw[h * 2 + warp] = b;
     }
     __syncthreads();
+    ig::Scaled<D> scaled;
     bool pend = (faces & (1 << kFaceFull)) != 0;
 #pragma unroll
     for (int w = 0; w < HW; ++w) pend = pend || (hm[w] & fl->hw[w]) != 0u;
@@ -207,7 +208,7 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
           side[2 * ax + 1] = t[ps + kStride[ax]];
           a[ax] = umin64(side[2 * ax], side[2 * ax + 1]);
         }
-        if (pend) did = hw::relax<D>(own, a, c, nv);
+        if (pend) did = hw::relax<D>(own, a, c, nv, nullptr, scaled);
         __syncwarp();
         if (did) {
           t[ps] = nv;
