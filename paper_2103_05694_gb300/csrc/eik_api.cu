@@ -399,13 +399,13 @@ bool use_guided(const eik_opts *o) {
 // and the guided kernel's fewer evaluations win (batches of 128^3 grids, front
 // against guided: 16.8 M cells 5.7 and 8.7 ms, 33.5 M 10.5 and 11.3, 67 M 20.8 and
 // 16.5, 185 M 58 and 36).  CTAs per SM: a single 2D front has few active tiles, and
-// more CTAs take tiles out of order (751 x 2301 section: 4 CTAs 4.1 ms, 8 4.9 ms,
-// 2 4.4 ms; 1502 x 4602: 9.4 ms, with 3 10.4 ms); elsewhere as many as fit (24
-// sections: 8 to 12 CTAs 1.9 ms, 16 2.3 ms; 256^3 checkerboard: 8 10.9 ms, 12 8.7,
+// more CTAs take tiles out of order (751 x 2301 section: 3 to 5 CTAs 3.3 ms, 6 3.2,
+// 8 3.5; 1502 x 4602: 9.5, 8.1, 7.6, 7.4 and 7.4 ms); elsewhere as many as fit (24
+// sections: 8 CTAs 1.66 ms, 10 1.55, 12 1.52, 16 with spills more; 256^3 checkerboard: 8 10.9 ms, 12 8.7,
 // 14 8.0, 20 with spills 9.3; 97 x 131 x 203: 12 1.76, 14 1.82, 16 2.1; many 3D
 // fronts launch the 20 of the other kernels, of which 14 run at a time).  Bucket
-// widths: the layered section 4.4 ms at 8, 4.2 at 16, 4.1 at 32; 32 sources of
-// 1024^2 11.0 ms at 2, 11.2 at 4, 11.6 at 16; 3D 1.80 ms (97 x 131 x 203) and 8.6 ms
+// widths: the layered section 4.4 ms at 8, 4.2 at 16, 4.1 at 32 (before the look
+// ahead); 32 sources of 1024^2 11.0 ms at 2, 11.2 at 4, 11.6 at 16; 3D 1.80 ms (97 x 131 x 203) and 8.6 ms
 // (checkerboard) at 0.4, 1.74 and 9.0 at 0.75, 1.75 and 9.7 at 1.5.
 struct GuidedCfg {
   int shape;
@@ -416,9 +416,19 @@ struct GuidedCfg {
 GuidedCfg guided_config(int ndim, int64_t total_sources, int64_t cells) {
   const bool many = total_sources >= kManyFronts;
   if (ndim == 2)
-    return many ? GuidedCfg{eik::kFrontShape, 4.0, 16, eik::kFrontCtas2} : GuidedCfg{eik::kFrontShape, 32.0, 16, 4};
+    return many ? GuidedCfg{eik::kFrontShape, 4.0, 16, eik::kFrontCtas2} : GuidedCfg{eik::kFrontShape, 32.0, 16, 6};
   if (many && cells >= int64_t(40) * 1000 * 1000) return GuidedCfg{eik::kGuidedShape0, 0.75, 31, eik::kGuidedCtas};
   return GuidedCfg{eik::kFrontShape, 0.5, 31, many ? eik::kGuidedCtas : eik::kFrontCtas3};
+}
+
+// Whether a 2D front kernel's CTAs outnumber the tiles that its fronts are in (about
+// 1.5 n^(1/2) for a problem of n tiles), so that tiles may start before a front
+// reaches them (measured in eik_front.cu).
+int front_ahead(const std::vector<Prob> &probs, int ndim, int shape, int64_t grid) {
+  if (ndim != 2 || shape != eik::kFrontShape) return 0;
+  double tiles = 0.0;
+  for (const Prob &P : probs) tiles += 1.5 * std::sqrt((double)(P.ntx * P.nty));
+  return tiles <= (double)grid ? 1 : 0;
 }
 
 // Tile shape of opts (validated): shape index and cells per axis.  opts.tile 0
@@ -875,6 +885,7 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
   int dev_sms = 0;
   CK(cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, ws().device), "SM count");
   const int64_t grid = size_grid(sp, opts, ndim, shape, tx * ty * tz, count_cells(hps), fronts, total_tiles, dev_sms);
+  sp.ahead = front_ahead(probs, ndim, shape, grid);
 
   eik_stats acc;
   std::memset(&acc, 0, sizeof(acc));
@@ -1169,9 +1180,11 @@ eik_status eik_autotune(const eik_problem *probs, int nprob, const eik_opts *bas
     if (std::memcmp(&start, &cur, sizeof(cur)) == 0) break;   // no change in a whole pass
   }
   if (st != EIK_OK) { if (ntrials) *ntrials = std::min(n, max_trials); return st; }
-  // the guided kernel against the best of the options above
+  // the front or guided kernel against the best of the options above (it has its
+  // own tiles: the first shape stands for none)
   eik_opts guided = cur;
   guided.arith = kArithGuided;
+  guided.tile = 1;
   if (use_guided(base) && use_guided(&guided)) {
     if ((st = consider(guided)) != EIK_OK) { if (ntrials) *ntrials = std::min(n, max_trials); return st; }
   }
@@ -1694,6 +1707,7 @@ eik_status plan_build(eik_plan &pl, std::vector<HostProblem> &hps, const eik_opt
   int sms = 0;
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, pl.device), "SM count");
   pl.grid = (int)size_grid(sp, opts, pl.ndim, shape, tx * ty * tz, count_cells(hps), pl.nseeds, pl.total_tiles, sms);
+  sp.ahead = front_ahead(pl.probs, pl.ndim, shape, pl.grid);
   return EIK_OK;
 }
 

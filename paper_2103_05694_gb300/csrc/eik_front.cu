@@ -34,7 +34,15 @@
 // kernel stays ahead (88-problem 3D batch: 57 against 135 ms).
 // One warp of two cells per lane: 5290 against 4086 us on the section (1.7
 // evaluations per round), but 7.6 against 8.0 ms on the checkerboard.
-// Polling a few rounds longer before a visit ends: no gain (5.25 -> 5.3 ms).
+// In 2D, where CTAs are free for it (SolveParams::ahead), a tile that a first front
+// reaches activates the neighbours that none has reached, and such a tile looks at
+// its halo for up to 16 rounds: starting a visit (push, pop, claim, loads: about 12
+// kcycles) then overlaps the front's way through the tile before (8 rounds of 1900;
+// a strip of 8 x 4096 cells 7.4 -> 5.7 ms, 129^2 252 -> 217 us, the section 3900 ->
+// 3180, 1502 x 4602 8980 -> 7360, 24 ragged sections 1724 -> 1520).  3D tiles are
+// reached from several sides, and the waiting CTAs are missed: checkerboard 7.6 ->
+// 8.6 ms, 97 x 131 x 203 1.68 -> 1.74; 32 sources of 1024^2 10.8 -> 11.3 ms.
+// Waiting a few rounds before any visit ends: no gain (5.25 -> 5.3 ms).
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -46,8 +54,10 @@
 namespace eik {
 namespace {
 
-template <int D>
+// AHEAD: see above (2D).
+template <int D, bool AHEAD>
 __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_kernel(SolveParams p) {
+  constexpr int kAhead = 16;           // rounds a tile waits for its first front
   constexpr int TX = D == 3 ? 4 : 8, TY = TX, TZ = D == 3 ? 4 : 1, HZ = D == 3 ? 1 : 0;
   constexpr int SX = TX + 2, SY = TY + 2, SZ = TZ + 2 * HZ, NS = SX * SY * SZ;
   constexpr int F = 64 / TX, H = 2 * D * F, HW = H / 32, HT = (H + 63) / 64;   // cells per face, halo cells, words, per thread
@@ -148,14 +158,21 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
                   z0 = static_cast<int64_t>(tcz) * TZ;
     const int64_t sy = nx, sz = nx * ny, first = z0 * sz + y0 * sy + x0;
     unsigned long long *const T0 = reinterpret_cast<unsigned long long *>(ldg_i64(&P.t)) + first;
-    // faces of this cell across which there is a tile
+    // the faces across which there is a tile, and those of them this cell lies on
+    const unsigned open_all = ((tcx > 0 ? 1u : 0u) | (tcx + 1 < ntx ? 2u : 0u) | (tcy > 0 ? 4u : 0u) |
+                                  (tcy + 1 < nty ? 8u : 0u) | (tcz > 0 ? 16u : 0u) | (tcz + 1 < ntz ? 32u : 0u));
     const unsigned open = edge & ((tcx > 0 ? 1u : 0u) | (tcx + 1 < ntx ? 2u : 0u) | (tcy > 0 ? 4u : 0u) |
                                   (tcy + 1 < nty ? 8u : 0u) | (tcz > 0 ? 16u : 0u) | (tcz + 1 < ntz ? 32u : 0u));
     const bool in = cc[0] < nx - x0 && cc[1] < ny - y0 && cc[2] < nz - z0;
     const int64_t off = cc[2] * sz + cc[1] * sy + cc[0];
     unsigned long long *const at = T0 + off;
     const unsigned long long c = in ? static_cast<unsigned long long>(ldg_i64(C0 + first + off)) : 0ull;
-    t[ps] = in ? ld_rlx(at) : kInfBits;
+    {
+      const unsigned long long v = in ? ld_rlx(at) : kInfBits;
+      t[ps] = v;
+      const unsigned b = __ballot_sync(kFull, v < kInfBits);
+      if (lane == 0) flags[0].chg[warp] = b;
+    }
     const bool fixed = !in || (p.tile_src[tile] != 0 && is_source(P, first + off));
     const unsigned long long *hat[HT];
     Round *fl = &flags[0];
@@ -176,6 +193,11 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
 #pragma unroll
     for (int w = 0; w < HW; ++w) pend = pend || (hm[w] & fl->hw[w]) != 0u;
     pend = pend && !fixed;
+    bool fresh = AHEAD && !(fl->chg[0] | fl->chg[1]);   // no front has reached the tile
+    unsigned fin[HW];                                   // halo cells that have a value
+#pragma unroll
+    for (int w = 0; w < HW; ++w) fin[w] = fl->hw[w];
+    int quiet = 0;
     unsigned notified = 0u, later = 0u;
     unsigned long long later_min = kInfBits;
     auto notify = [&](unsigned set, unsigned long long min) {    // warp 0
@@ -187,6 +209,32 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
       }
       __syncwarp();
     };
+    // the first front reaches the tile: the tiles that it has not reached either start
+    // now, and look for it while it crosses this one
+    auto wake = [&]() {
+      unsigned set = 0u;
+#pragma unroll
+      for (int j = 0; j < 2 * D; ++j)
+        if (!((fin[j * F / 32] >> (j * F % 32)) & ((1u << F) - 1u))) set |= 1u << j;
+      set &= open_all;
+      if (set && warp == 0) {
+        unsigned long long m = kInfBits;      // the smallest halo value
+#pragma unroll
+        for (int w = 0; w < HW; ++w) {
+          const int i = w * 32 + lane, j = i / F, n = i % F, ax = j >> 1, e = (j & 1) ? TX : -1;
+          m = umin64(m, t[pos_of(ax == 0 ? e : n % TX, ax == 0 ? n % TY : ax == 1 ? e : n / TX,
+                                 ax == 2 ? e : D == 3 ? n / TX : 0)]);
+        }
+        notify(set, warp_min64(m));
+      }
+      notified |= set;
+    };
+    if (fresh) {
+      unsigned a = 0u;
+#pragma unroll
+      for (int w = 0; w < HW; ++w) a |= fin[w];
+      if (a) { wake(); fresh = false; }
+    }
 #pragma unroll 1
     for (unsigned round = 0;; ++round) {
       if (round >= kMaxRounds) {
@@ -254,7 +302,14 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
         if (now && warp == 0) notify(now, m);
         notified |= now;
       }
-      if (any) continue;
+      if (fresh) {
+        unsigned a = 0u;
+#pragma unroll
+        for (int w = 0; w < HW; ++w) a |= (fin[w] |= fl->hw[w]);
+        if (a) { wake(); fresh = false; }
+      }
+      if (any) { quiet = 0; continue; }
+      if (fresh && ++quiet <= kAhead) continue;
       // done, unless the tile was re-activated meanwhile
       if (warp == 0) {
         if (later) notify(later, later_min);
@@ -294,8 +349,9 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
 
 cudaError_t launch_front(const SolveParams &p, int grid, cudaStream_t stream) {
   note_launches(1);
-  if (p.ndim == 2) front_kernel<2><<<grid, 64, 0, stream>>>(p);
-  else front_kernel<3><<<grid, 64, 0, stream>>>(p);
+  if (p.ndim == 3) front_kernel<3, false><<<grid, 64, 0, stream>>>(p);
+  else if (p.ahead) front_kernel<2, true><<<grid, 64, 0, stream>>>(p);
+  else front_kernel<2, false><<<grid, 64, 0, stream>>>(p);
   return cudaGetLastError();
 }
 

@@ -88,6 +88,7 @@ struct SolveParams {
                                   // the last visit (to evaluate at the next one)
   unsigned long long *slots;      // kNumSlots * cap
   unsigned cap_mask;              // cap - 1
+  int ahead;                      // front kernel: activate tiles before a first front reaches them
   Ctl *ctl;
   long long timeout_ns;
   int counters;

@@ -83,3 +83,19 @@ def test_large_batches_equal_the_tile_kernel(n):
         eik.eik_solve_batched([{"speed": speed, "h": p.h, "sources": s, "out": t} for s, t in zip(srcs, o)], opts)
     for a, b in zip(*outs):
         assert torch.equal(a.view(torch.int64), b.view(torch.int64))
+
+
+@pytest.mark.parametrize("n_grids", [1, 40])
+def test_look_ahead_in_2d(n_grids):
+    """Few grids: tiles start before a front reaches them.  Many: they don't (their
+    fronts are in more tiles than there are CTAs).  Slow walls keep fronts away
+    from tiles that wait for them."""
+    speed = np.full((420, 600), 1.0)
+    speed[::24, 5:] = speed[12::24, :-5] = 1e-4
+    ref = oracle.fmm(speed, 0.5, [7]).t
+    dev = _dev(speed)
+    probs = [{"speed": dev, "h": 0.5, "sources": torch.tensor([7], device=DEV), "out": torch.empty_like(dev)}
+             for _ in range(n_grids)]
+    eik.eik_solve_batched(probs)
+    for q in probs:
+        assert np.array_equal(q["out"].cpu().numpy().view(np.uint64), ref.view(np.uint64))
