@@ -423,12 +423,14 @@ GuidedCfg guided_config(int ndim, int64_t total_sources, int64_t cells) {
 
 // Whether a 2D front kernel's CTAs outnumber the tiles that its fronts are in (about
 // 1.5 n^(1/2) for a problem of n tiles), so that tiles may start before a front
-// reaches them (measured in eik_front.cu).
-int front_ahead(const std::vector<Prob> &probs, int ndim, int shape, int64_t grid) {
+// reaches them: 1; 2 with few fronts, whose 6 CTAs per SM have room for a warp more
+// (measured in eik_front.cu).
+int front_ahead(const std::vector<Prob> &probs, int ndim, int shape, bool many, int64_t grid) {
   if (ndim != 2 || shape != eik::kFrontShape) return 0;
   double tiles = 0.0;
   for (const Prob &P : probs) tiles += 1.5 * std::sqrt((double)(P.ntx * P.nty));
-  return tiles <= (double)grid ? 1 : 0;
+  if (tiles > (double)grid) return 0;
+  return many ? 1 : 2;
 }
 
 // Tile shape of opts (validated): shape index and cells per axis.  opts.tile 0
@@ -885,7 +887,7 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
   int dev_sms = 0;
   CK(cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, ws().device), "SM count");
   const int64_t grid = size_grid(sp, opts, ndim, shape, tx * ty * tz, count_cells(hps), fronts, total_tiles, dev_sms);
-  sp.ahead = front_ahead(probs, ndim, shape, grid);
+  sp.ahead = front_ahead(probs, ndim, shape, fronts >= kManyFronts, grid);
 
   eik_stats acc;
   std::memset(&acc, 0, sizeof(acc));
@@ -1707,7 +1709,7 @@ eik_status plan_build(eik_plan &pl, std::vector<HostProblem> &hps, const eik_opt
   int sms = 0;
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, pl.device), "SM count");
   pl.grid = (int)size_grid(sp, opts, pl.ndim, shape, tx * ty * tz, count_cells(hps), pl.nseeds, pl.total_tiles, sms);
-  sp.ahead = front_ahead(pl.probs, pl.ndim, shape, pl.grid);
+  sp.ahead = front_ahead(pl.probs, pl.ndim, shape, pl.nseeds >= kManyFronts, pl.grid);
   return EIK_OK;
 }
 

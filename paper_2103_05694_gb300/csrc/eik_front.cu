@@ -42,6 +42,11 @@
 // 3180, 1502 x 4602 8980 -> 7360, 24 ragged sections 1724 -> 1520).  3D tiles are
 // reached from several sides, and the waiting CTAs are missed: checkerboard 7.6 ->
 // 8.6 ms, 97 x 131 x 203 1.68 -> 1.74; 32 sources of 1024^2 10.8 -> 11.3 ms.
+// With few fronts a third warp activates the neighbours (an activation is a fence
+// and three dependent atomics, 5 kcycles, about 1.5 times a visit), so that the rounds
+// go on meanwhile: 129^2 219 -> 205 us, the section 3150 -> 3030, 1502 x 4602 7360 ->
+// 6700.  It also claims the tiles and ends the visits; its mailbox takes the bucket
+// time of each face.
 // Waiting a few rounds before any visit ends: no gain (5.25 -> 5.3 ms).
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -54,9 +59,10 @@
 namespace eik {
 namespace {
 
-// AHEAD: see above (2D).
-template <int D, bool AHEAD>
-__global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_kernel(SolveParams p) {
+// AHEAD, HELP (2D): see above.
+template <int D, bool AHEAD, bool HELP>
+__global__ void __launch_bounds__(HELP ? 96 : 64, HELP ? kFrontCtasHelp : D == 3 ? kFrontCtas3 : kFrontCtas2)
+    front_kernel(SolveParams p) {
   constexpr int kAhead = 16;           // rounds a tile waits for its first front
   constexpr int TX = D == 3 ? 4 : 8, TY = TX, TZ = D == 3 ? 4 : 1, HZ = D == 3 ? 1 : 0;
   constexpr int SX = TX + 2, SY = TY + 2, SZ = TZ + 2 * HZ, NS = SX * SY * SZ;
@@ -72,6 +78,8 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
   __shared__ unsigned long long sh_tile;
   __shared__ unsigned sh_lo, sh_slot;
   __shared__ int sh_faces;
+  __shared__ unsigned long long mail[4];       // HELP: bucket time of a face to activate, kEmpty: none
+  __shared__ volatile int sh_fin;              // HELP: the rounds are over
   volatile unsigned long long *const t = t_mem;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float inv_delta = static_cast<float>(p.ctl->inv_delta);
@@ -107,9 +115,15 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
     hps[c] = i < H ? pos_of(hc[c][0], hc[c][1], hc[c][2]) : 0;
   }
 
+  auto sync_rounds = [] {                      // the warps that hold cells
+    if (HELP) asm volatile("bar.sync 1, 64;" ::: "memory");
+    else __syncthreads();
+  };
+  if (HELP && tid < 4) mail[tid] = kEmpty;
+  if (HELP && tid == 0) sh_fin = 0;
 #pragma unroll 1
   for (;;) {
-    if (warp == 0) {
+    if (warp == (HELP ? 2 : 0)) {
       unsigned slot = 0, lo = 0;
       unsigned long long tile = kEmpty;
       int faces = 0;
@@ -163,6 +177,66 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
                                   (tcy + 1 < nty ? 8u : 0u) | (tcz > 0 ? 16u : 0u) | (tcz + 1 < ntz ? 32u : 0u));
     const unsigned open = edge & ((tcx > 0 ? 1u : 0u) | (tcx + 1 < ntx ? 2u : 0u) | (tcy > 0 ? 4u : 0u) |
                                   (tcy + 1 < nty ? 8u : 0u) | (tcz > 0 ? 16u : 0u) | (tcz + 1 < ntz ? 32u : 0u));
+    auto activate_faces = [&](unsigned set, unsigned long long min) {
+      if ((set >> lane) & 1u) {
+        fence_ar();
+        const int64_t step = (lane >> 1) == 0 ? 1 : (lane >> 1) == 1 ? ntx : static_cast<int64_t>(ntx) * nty;
+        activate(p, static_cast<unsigned long long>(tile + ((lane & 1) ? step : -step)), 1u << (lane ^ 1),
+                 bucket_of_time(min, inv_delta), lo);
+      }
+      __syncwarp();
+    };
+    // done, unless the tile was re-activated meanwhile (one thread)
+    auto finish = [&] {
+      int cont = 0;
+      const unsigned long long mine = make_state(kStRunning, 0, 0);
+      unsigned long long old = mine;
+#pragma unroll 1
+      for (int it = 0;; ++it) {
+        const unsigned long long prev = atomicCAS(&p.state[tile], old, old == mine ? 0ull : mine);
+        if (prev == old) {
+          cont = old != mine;
+          break;
+        }
+        old = prev;
+        if (it > (1 << 22)) { raise_status(p.ctl, kEtimeout, 5); break; }
+      }
+      fence_ar();   // the claim of the new work before the halo loads; else the pushes'
+                    // work counts before this visit's
+      sh_faces = cont;
+    };
+    if (HELP && warp == 2) {
+#pragma unroll 1
+      for (;;) {
+        long long t0 = 0;
+#pragma unroll 1
+        for (unsigned it = 0;; ++it) {
+          const bool fin = sh_fin != 0;
+          __threadfence_block();
+          const unsigned long long m = lane < 4 ? atomicExch(&mail[lane], kEmpty) : kEmpty;
+          if (__any_sync(kFull, m != kEmpty)) {
+            activate_faces(m != kEmpty ? 1u << lane : 0u, m);
+            continue;
+          }
+          if (__all_sync(kFull, fin)) break;
+          if ((it & 255u) == 255u) {
+            const long long now = now_ns();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > p.timeout_ns) { if (lane == 0) raise_status(p.ctl, kEtimeout, 8); break; }
+          }
+          __nanosleep(20);
+        }
+        __syncwarp();
+        if (lane == 0) {
+          finish();
+          sh_fin = 0;
+        }
+        __syncthreads();
+        if (!sh_faces) break;
+      }
+      __syncthreads();
+      continue;
+    }
     const bool in = cc[0] < nx - x0 && cc[1] < ny - y0 && cc[2] < nz - z0;
     const int64_t off = cc[2] * sz + cc[1] * sy + cc[0];
     unsigned long long *const at = T0 + off;
@@ -187,7 +261,7 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
       const unsigned b = __ballot_sync(kFull, v < kInfBits);
       if (lane == 0) fl->hw[h * 2 + warp] = b;
     }
-    __syncthreads();
+    sync_rounds();
     ig::Scaled<D> scaled;
     bool pend = (faces & (1 << kFaceFull)) != 0;
 #pragma unroll
@@ -201,13 +275,15 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
     unsigned notified = 0u, later = 0u;
     unsigned long long later_min = kInfBits;
     auto notify = [&](unsigned set, unsigned long long min) {    // warp 0
-      if ((set >> lane) & 1u) {
-        fence_ar();
-        const int64_t step = (lane >> 1) == 0 ? 1 : (lane >> 1) == 1 ? ntx : static_cast<int64_t>(ntx) * nty;
-        activate(p, static_cast<unsigned long long>(tile + ((lane & 1) ? step : -step)), 1u << (lane ^ 1),
-                 bucket_of_time(min, inv_delta), lo);
+      if constexpr (HELP) {
+        if ((set >> lane) & 1u) {
+          __threadfence_block();
+          atomicExch(&mail[lane & 3], min);
+        }
+        __syncwarp();
+      } else {
+        activate_faces(set, min);
       }
-      __syncwarp();
     };
     // the first front reaches the tile: the tiles that it has not reached either start
     // now, and look for it while it crosses this one
@@ -239,7 +315,7 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
     for (unsigned round = 0;; ++round) {
       if (round >= kMaxRounds) {
         if (tid == 0) raise_status(p.ctl, kEtimeout, 7);
-        break;
+        if (!HELP) break;
       }
       unsigned long long hv[HT];
 #pragma unroll
@@ -283,7 +359,7 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
         const unsigned b = __ballot_sync(kFull, fell);
         if (lane == 0) fl->hw[h * 2 + warp] = b;
       }
-      __syncthreads();
+      sync_rounds();
       const unsigned long long chg = (static_cast<unsigned long long>(fl->chg[1]) << 32) | fl->chg[0];
       unsigned any = fl->chg[0] | fl->chg[1];
       pend = (nb & chg) != 0ull;
@@ -308,28 +384,15 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
         for (int w = 0; w < HW; ++w) a |= (fin[w] |= fl->hw[w]);
         if (a) { wake(); fresh = false; }
       }
-      if (any) { quiet = 0; continue; }
+      if (any && (!HELP || round < kMaxRounds)) { quiet = 0; continue; }
       if (fresh && ++quiet <= kAhead) continue;
-      // done, unless the tile was re-activated meanwhile
       if (warp == 0) {
         if (later) notify(later, later_min);
-        if (lane == 0) {
-          int cont = 0;
-          const unsigned long long mine = make_state(kStRunning, 0, 0);
-          unsigned long long old = mine;
-#pragma unroll 1
-          for (int it = 0;; ++it) {
-            const unsigned long long prev = atomicCAS(&p.state[tile], old, old == mine ? 0ull : mine);
-            if (prev == old) {
-              cont = old != mine;
-              break;
-            }
-            old = prev;
-            if (it > (1 << 22)) { raise_status(p.ctl, kEtimeout, 5); break; }
-          }
-          fence_ar();   // the claim of the new work before the halo loads; else the pushes'
-                        // work counts before this visit's
-          sh_faces = cont;
+        if (HELP) {
+          __threadfence_block();
+          if (lane == 0) sh_fin = 1;
+        } else if (lane == 0) {
+          finish();
         }
       }
       later = 0u;
@@ -349,9 +412,10 @@ __global__ void __launch_bounds__(64, D == 3 ? kFrontCtas3 : kFrontCtas2) front_
 
 cudaError_t launch_front(const SolveParams &p, int grid, cudaStream_t stream) {
   note_launches(1);
-  if (p.ndim == 3) front_kernel<3, false><<<grid, 64, 0, stream>>>(p);
-  else if (p.ahead) front_kernel<2, true><<<grid, 64, 0, stream>>>(p);
-  else front_kernel<2, false><<<grid, 64, 0, stream>>>(p);
+  if (p.ndim == 3) front_kernel<3, false, false><<<grid, 64, 0, stream>>>(p);
+  else if (p.ahead == 2) front_kernel<2, true, true><<<grid, 96, 0, stream>>>(p);
+  else if (p.ahead) front_kernel<2, true, false><<<grid, 64, 0, stream>>>(p);
+  else front_kernel<2, false, false><<<grid, 64, 0, stream>>>(p);
   return cudaGetLastError();
 }
 

@@ -88,7 +88,8 @@ struct SolveParams {
                                   // the last visit (to evaluate at the next one)
   unsigned long long *slots;      // kNumSlots * cap
   unsigned cap_mask;              // cap - 1
-  int ahead;                      // front kernel: activate tiles before a first front reaches them
+  int ahead;                      // front kernel: 1: activate tiles before a first front reaches
+                                  // them, 2: and leave activations to a warp of their own
   Ctl *ctl;
   long long timeout_ns;
   int counters;
@@ -156,7 +157,7 @@ struct TileShape {
 constexpr int kGuidedShape0 = kNumTileShapes;       // 8x8x4, one warp per tile
 constexpr int kFrontShape = kNumTileShapes + 1;     // 8x8, 4x4x4, a thread per cell
 constexpr int kGuidedCtas = 20;
-constexpr int kFrontCtas2 = 12, kFrontCtas3 = 14;
+constexpr int kFrontCtas2 = 12, kFrontCtas3 = 14, kFrontCtasHelp = 6;
 __host__ __device__ inline TileShape tile_shape_of(int ndim, int shape) {
   if (shape == kGuidedShape0) return TileShape{8, 8, 4};
   if (shape == kFrontShape) return ndim == 3 ? TileShape{4, 4, 4} : TileShape{8, 8, 1};
