@@ -51,20 +51,19 @@ METRIC = "useful grid-point updates/s and % HBM roofline (bit-exact vs FP64 FMM 
 UNIT = "updates/s"
 B_ALG = 24          # algorithmic bytes per useful update: read c once, read t once, write t once
 L2_FLUSH_BYTES = 512 << 20
-# ncu DRAM bytes (read + write) per launch of the persistent kernel in its default
+# ncu DRAM bytes (read + write) per launch of the tile kernel in its default
 # configuration (the instantiation the timed steps run), from the one-pass
 # captures summarised in profiles/ (refresh them whenever the kernel changes)
-MEASURED_TRAFFIC = {"layered_2d": 28089088 + 668416, "checker_3d": 283825920 + 117156352}
+MEASURED_TRAFFIC = {"layered_2d": 28283648 + 3198464, "checker_3d": 276162048 + 114629120}
 # ncu DRAM bytes of one launch of the 88-problem batch in the default options
 # (the benchmark autotunes, so this is context, not the traffic of the timed launch)
-BATCH_TRAFFIC_DEFAULT_OPTIONS = 16199321088 + 2499080704
+BATCH_TRAFFIC_DEFAULT_OPTIONS = 15417601280 + 2447531776
 
 # FP64 thread instructions (DADD + DMUL + DFMA, ncu sass counters) per operator
-# evaluation of the persistent kernel, by dimension, from one-launch captures of
-# the counting instantiation (whose evaluation count comes from the same launch;
-# the timed instantiation runs the same d-bar code), summarised in profiles/
-# (refresh them whenever the kernel changes)
-MEASURED_FP64_PER_EVAL = {2: 8.031, 3: 12.982, "batched_3d": 12.717}
+# evaluation, by dimension or workload.  None apply to the default kernels: they
+# evaluate d-bar on the integer and FP32 pipes but for the cells that need exact
+# values of G, and have no counting build to relate the instructions to.
+MEASURED_FP64_PER_EVAL = {}
 
 WORKLOADS = {
     "layered_2d": "2d_2301x751_layered_h4_1src",
@@ -438,7 +437,7 @@ def roofline(useful_per_launch: int, kern_ms: float, traffic, what: str):
 
 def roofline_fp64(C, evals_per_launch: int, kern_ms: float, ndim: int, what: str,
                   workload: str | None = None):
-    """The FP64 roofline of the persistent kernel: FP64 thread instructions per
+    """The FP64 roofline of the tile kernel: FP64 thread instructions per
     launch (ncu instructions per evaluation x the live evaluation count) over the
     kernel's event time, against the device's measured FP64 add rate."""
     per_eval = MEASURED_FP64_PER_EVAL.get(workload, MEASURED_FP64_PER_EVAL.get(ndim))
@@ -570,7 +569,7 @@ def run_single(args, C, wl_name):
     if traffic is None and not opts and args.scale == 1.0 and args.upsample == 1 and not args.autotune:
         traffic = MEASURED_TRAFFIC.get(args.workload)
     line["roofline"] = roofline(useful, statistics.mean(solve_ms), traffic,
-                                ["persistent_kernel (tile relaxation + bucket scheduler)",
+                                ["tile kernel (relaxation + bucket scheduler)",
                                  "fim_kernel (Algorithm 3 rounds)",
                                  "topo_kernel (Algorithm 4 iterations)",
                                  "fsm_kernel (Algorithm 5 sweeps)"][args.schedule])
@@ -685,7 +684,7 @@ def run_batched(args, C, wl_name):
     line["work_per_step"].update(empty=st["evals"] - st["decreases"],
                                  bad=st["decreases"] - st["good"])
     line["roofline"] = roofline(useful_mine, statistics.mean(solve_ms), args.traffic_bytes,
-                                "persistent_kernel (all problems in one launch)")
+                                "tile kernel (all problems in one launch)")
     if args.problems == 0:
         line["roofline"]["traffic_default_options"] = BATCH_TRAFFIC_DEFAULT_OPTIONS
     line["roofline_fp64"] = roofline_fp64(C, st["evals"], statistics.mean(solve_ms), 3,
@@ -816,7 +815,7 @@ def run_tomography(args, C, wl_name):
                           "speedup_vs_per_source": (per_source_ms / (total_ms / args.steps)
                                                     if per_source_ms else None)}
     line["roofline"] = roofline(len(srcs) * (s0.numel() - 1), statistics.mean(solve_ms),
-                                args.traffic_bytes, "persistent_kernel (batched forward)")
+                                args.traffic_bytes, "tile kernel (batched forward)")
     line["roofline_fp64"] = roofline_fp64(C, fwd_evals, statistics.mean(solve_ms), 2,
                                           line["roofline"]["kernel"])
     line["e2e"] = {"value": useful_all / (e2e_ms / 1e3), "unit": UNIT, "ms_per_step": e2e_ms,
