@@ -424,13 +424,18 @@ GuidedCfg guided_config(int ndim, int64_t total_sources, int64_t cells) {
 // Whether a 2D front kernel's CTAs outnumber the tiles that its fronts are in (about
 // 1.5 n^(1/2) for a problem of n tiles), so that tiles may start before a front
 // reaches them: 1; 2 with few fronts, whose 6 CTAs per SM have room for a warp more
-// (measured in eik_front.cu).
-int front_ahead(const std::vector<Prob> &probs, int ndim, int shape, bool many, int64_t grid) {
+// (measured in eik_front.cu).  Else 0, and more CTAs share the tiles (32 sources of
+// 1024^2: 12 per SM 10.7 ms, 14 10.4, 16 10.0, 18 10.1; with the look ahead and 6 or
+// 12 per SM against without and 16: one 8000^2 section 37.3 and 31.0 ms, five of
+// 3000^2 27.6 and 17.0, three of 1502 x 4602 12.9 and 12.4).
+int front_ahead(const std::vector<Prob> &probs, int ndim, int shape, bool many, int sms, int64_t total_tiles,
+                int64_t &grid) {
   if (ndim != 2 || shape != eik::kFrontShape) return 0;
   double tiles = 0.0;
   for (const Prob &P : probs) tiles += 1.5 * std::sqrt((double)(P.ntx * P.nty));
-  if (tiles > (double)grid) return 0;
-  return many ? 1 : 2;
+  if (tiles <= (double)grid) return many ? 1 : 2;
+  grid = std::min<int64_t>((int64_t)sms * eik::kFrontCtasMany2, total_tiles);
+  return 0;
 }
 
 // Tile shape of opts (validated): shape index and cells per axis.  opts.tile 0
@@ -886,8 +891,8 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
      "seed launch");
   int dev_sms = 0;
   CK(cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, ws().device), "SM count");
-  const int64_t grid = size_grid(sp, opts, ndim, shape, tx * ty * tz, count_cells(hps), fronts, total_tiles, dev_sms);
-  sp.ahead = front_ahead(probs, ndim, shape, fronts >= kManyFronts, grid);
+  int64_t grid = size_grid(sp, opts, ndim, shape, tx * ty * tz, count_cells(hps), fronts, total_tiles, dev_sms);
+  sp.ahead = front_ahead(probs, ndim, shape, fronts >= kManyFronts, dev_sms, total_tiles, grid);
 
   eik_stats acc;
   std::memset(&acc, 0, sizeof(acc));
@@ -1708,8 +1713,9 @@ eik_status plan_build(eik_plan &pl, std::vector<HostProblem> &hps, const eik_opt
   pl.from_slowness = from_slowness(opts);
   int sms = 0;
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, pl.device), "SM count");
-  pl.grid = (int)size_grid(sp, opts, pl.ndim, shape, tx * ty * tz, count_cells(hps), pl.nseeds, pl.total_tiles, sms);
-  sp.ahead = front_ahead(pl.probs, pl.ndim, shape, pl.nseeds >= kManyFronts, pl.grid);
+  int64_t grid = size_grid(sp, opts, pl.ndim, shape, tx * ty * tz, count_cells(hps), pl.nseeds, pl.total_tiles, sms);
+  sp.ahead = front_ahead(pl.probs, pl.ndim, shape, pl.nseeds >= kManyFronts, sms, pl.total_tiles, grid);
+  pl.grid = (int)grid;
   return EIK_OK;
 }
 

@@ -61,7 +61,7 @@ namespace {
 
 // AHEAD, HELP (2D): see above.
 template <int D, bool AHEAD, bool HELP>
-__global__ void __launch_bounds__(HELP ? 96 : 64, HELP ? kFrontCtasHelp : D == 3 ? kFrontCtas3 : kFrontCtas2)
+__global__ void __launch_bounds__(HELP ? 96 : 64, HELP ? kFrontCtasHelp : D == 3 ? kFrontCtas3 : AHEAD ? kFrontCtas2 : kFrontCtasMany2)
     front_kernel(SolveParams p) {
   constexpr int kAhead = 16;           // rounds a tile waits for its first front
   constexpr int TX = D == 3 ? 4 : 8, TY = TX, TZ = D == 3 ? 4 : 1, HZ = D == 3 ? 1 : 0;

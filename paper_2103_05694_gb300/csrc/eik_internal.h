@@ -157,7 +157,7 @@ struct TileShape {
 constexpr int kGuidedShape0 = kNumTileShapes;       // 8x8x4, one warp per tile
 constexpr int kFrontShape = kNumTileShapes + 1;     // 8x8, 4x4x4, a thread per cell
 constexpr int kGuidedCtas = 20;
-constexpr int kFrontCtas2 = 12, kFrontCtas3 = 14, kFrontCtasHelp = 6;
+constexpr int kFrontCtas2 = 12, kFrontCtasMany2 = 16, kFrontCtas3 = 14, kFrontCtasHelp = 6;
 __host__ __device__ inline TileShape tile_shape_of(int ndim, int shape) {
   if (shape == kGuidedShape0) return TileShape{8, 8, 4};
   if (shape == kFrontShape) return ndim == 3 ? TileShape{4, 4, 4} : TileShape{8, 8, 1};

@@ -85,10 +85,10 @@ def test_large_batches_equal_the_tile_kernel(n):
         assert torch.equal(a.view(torch.int64), b.view(torch.int64))
 
 
-@pytest.mark.parametrize("n_grids", [1, 40])
+@pytest.mark.parametrize("n_grids", [1, 7, 12, 40])
 def test_look_ahead_in_2d(n_grids):
     """Few grids: tiles start before a front reaches them.  Many: they don't (their
-    fronts are in more tiles than there are CTAs).  Slow walls keep fronts away
+    fronts are in more tiles than there are CTAs), and more CTAs share the tiles.  Slow walls keep fronts away
     from tiles that wait for them."""
     speed = np.full((420, 600), 1.0)
     speed[::24, 5:] = speed[12::24, :-5] = 1e-4
