@@ -290,15 +290,17 @@ eik_status eik_solve_noalloc(const double *speed, double h, int ndim, const int6
  * reproducible bit for bit.  Device pointers only.  A parallel set-up pass
  * evaluates every weight; then the cells are processed in dependency order by
  * one of two schedules (opts->sched_flags bits 3-4), with the same results:
- *   tiles (default): persistent CTAs take tiles of 16x8 (2D) or 8x8x4 (3D)
- *     cells from a queue and run the dependency order inside a tile in shared
- *     memory; a tile is queued when a cell of it may have become ready;
+ *   tiles (default): persistent warps take tiles of 16x16 (2D) or 8x4x4 (3D)
+ *     cells, latest times first, and run the dependency order inside a tile in
+ *     shared memory; a tile is queued when a cell of it may have become ready;
  *   levels: one cooperative launch processes the cells level by level, its
  *     blocks meeting at a grid barrier between levels.
  * Every device wait is bounded by opts->timeout_ms (EIK_ETIMEOUT); opts->
- * ctas_per_sm caps the CTAs of the tile schedule.  Workspace: about 34 (tiles)
- * or 53 (levels) bytes per cell of the batch, kept for the next call
- * (eik_release frees it).
+ * ctas_per_sm caps the CTAs of the tile schedule (0: chosen by the size of the
+ * fronts).  Workspace: about 18 to 30 (tiles; 8 more for models
+ * that problems share) or 53 (levels) bytes per cell of the batch, kept for the
+ * next call (eik_release frees it).  EIK_ECAPACITY: the tile schedule's frontier
+ * outgrew four entries per tile and bucket.
  * Synchronises `stream`.  stats (optional): good = cells processed, evals =
  * reached cells, solve_ms = device time of the adjoint launches; tiles: visits
  * = tile visits, rounds = in-tile rounds summed over visits, ctas; with
@@ -322,10 +324,10 @@ eik_status eik_adjoint(const eik_problem *probs, int nprob, const double *const 
  * the epochs repeat until no exchanged value changes (a global AND over the
  * boundaries).  Ghost values only decrease from epoch to epoch, so the loop
  * ends, and then every cell satisfies the update with its neighbours' final
- * values: the union is the unique fixed point (Theorem 1).  Every epoch
- * solves the slabs from +inf; all slabs run on the calling device (with one
- * slab per GPU, the exchange is a peer copy of one row into the neighbour's
- * memory).
+ * values: the union is the unique fixed point (Theorem 1).  An epoch goes on
+ * from the last one's fields and solves the fronts that the lowered ghosts send
+ * out; all slabs run on the calling device (with one slab per GPU, the exchange
+ * is a peer copy of one row into the neighbour's memory).
  *   speed, out_t: device pointers; src_idx / src_t: host or device; other
  *   arguments as eik_solve.  1 <= nslabs <= outermost extent (EIK_EINVAL
  *   otherwise); opts->update, schedule, test_stall and sched_flags bit 5 must
