@@ -187,24 +187,7 @@ __global__ void __launch_bounds__(HELP ? 96 : 64, HELP ? kFrontCtasHelp : D == 3
       __syncwarp();
     };
     // done, unless the tile was re-activated meanwhile (one thread)
-    auto finish = [&] {
-      int cont = 0;
-      const unsigned long long mine = make_state(kStRunning, 0, 0);
-      unsigned long long old = mine;
-#pragma unroll 1
-      for (int it = 0;; ++it) {
-        const unsigned long long prev = atomicCAS(&p.state[tile], old, old == mine ? 0ull : mine);
-        if (prev == old) {
-          cont = old != mine;
-          break;
-        }
-        old = prev;
-        if (it > (1 << 22)) { raise_status(p.ctl, kEtimeout, 5); break; }
-      }
-      fence_ar();   // the claim of the new work before the halo loads; else the pushes'
-                    // work counts before this visit's
-      sh_faces = cont;
-    };
+    auto finish = [&] { sh_faces = end_visit(p, static_cast<unsigned long long>(tile)); };
     if (HELP && warp == 2) {
 #pragma unroll 1
       for (;;) {

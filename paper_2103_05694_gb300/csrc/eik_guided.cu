@@ -400,8 +400,8 @@ __global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) 
           if (lane == j) mine = v;
           fm_any |= 1u << j;
         }
-        fence_ar();
         __syncwarp();
+        fence_ar();               // every lane's stores before the activations
         if ((fm_any >> lane) & 1u) {
           const int ax = lane >> 1, up = lane & 1;
           const unsigned at = ax == 0 ? tcx : ax == 1 ? tcy : tcz, ext = ax == 0 ? ntx : ax == 1 ? nty : ntz;
@@ -416,28 +416,13 @@ __global__ void __launch_bounds__(32, kGuidedCtas) guided_kernel(SolveParams p) 
       // done, unless the tile was re-activated meanwhile: then go on with its new
       // faces
       int cont = 0;
-      if (lane == 0) {
-        const unsigned long long mine = make_state(kStRunning, 0, 0);
-        unsigned long long old = mine;
-#pragma unroll 1
-        for (int it = 0;; ++it) {
-          const unsigned long long prev = atomicCAS(&p.state[tile], old, old == mine ? 0ull : mine);
-          if (prev == old) {
-            if (old != mine) cont = 0x100 | static_cast<int>(faces_of(old));
-            break;
-          }
-          old = prev;
-          if (it > (1 << 22)) { raise_status(p.ctl, kEtimeout, 5); break; }
-        }
-        if (cont) fence_ar();   // the claim of the new work before the halo loads
-      }
+      if (lane == 0) cont = end_visit(p, static_cast<unsigned long long>(tile));
       cont = __shfl_sync(kFull, cont, 0);
       if (!cont) break;
       faces = cont & 0x7f;
     }
 
     if (lane == 0) {
-      fence_ar();                // the pushes' work counts before this visit's
       atomicAdd(&p.ctl->run[slot * kCounterPad], 0xffffffffu);
       atomicAdd(&p.ctl->work, -1);
     }

@@ -262,6 +262,30 @@ EIK_SCHED_FN void finish_tile(const SolveParams &p, unsigned long long tile) {
   raise_status(p.ctl, kEtimeout, 5);
 }
 
+// The same for the kernels that go on with a tile at once when it was re-activated
+// meanwhile: running -> idle (returns 0), or dirty -> running (0x100 | the new
+// faces).  One thread, after a barrier with the threads that stored the tile's
+// cells.  The fence makes the state a release of all of these stores: the next
+// visitor loads the cells with relaxed loads and stores over them, so a value that
+// it missed would be lost.
+__device__ __forceinline__ int end_visit(const SolveParams &p, unsigned long long tile) {
+  fence_ar();
+  const unsigned long long mine = make_state(kStRunning, 0, 0);
+  unsigned long long old = mine;
+#pragma unroll 1
+  for (int it = 0; it < (1 << 22); ++it) {
+    const unsigned long long prev = atomicCAS(&p.state[tile], old, old == mine ? 0ull : mine);
+    if (prev == old) {
+      if (old == mine) return 0;
+      fence_ar();   // the claim of the new work before the halo loads
+      return 0x100 | static_cast<int>(faces_of(old));
+    }
+    old = prev;
+  }
+  raise_status(p.ctl, kEtimeout, 5);
+  return 0;
+}
+
 // The entry at index q of slot s (reserved by the caller), freeing its position:
 // waits until a pusher has written it.  (If laps meet at a position, the
 // entries go to either taker: they are all live.)
