@@ -398,6 +398,10 @@ __device__ __forceinline__ unsigned ld_rlx_u8(const unsigned char *p) {
   return v;
 }
 
+__device__ __forceinline__ void st_rlx_u8(unsigned char *p, unsigned v) {
+  asm volatile("st.relaxed.gpu.global.u8 [%0], %1;" ::"l"(p), "h"(static_cast<unsigned short>(v)) : "memory");
+}
+
 __device__ __forceinline__ int find_tile_prob(const AdjProb *probs, int nprob, unsigned tile) {
   int lo = 0, hi = nprob - 1;
   while (lo < hi) {
@@ -667,11 +671,11 @@ __global__ void __launch_bounds__(32, kAdjCtas) adj_tiles_kernel(const AdjProb *
         if (!((w >> lane) & 1u)) continue;
         const int q = k * 32 + lane;
         const int64_t off = (q / (TX * TY)) * sz + ((q / TX) % TY) * sy + q % TX;
-        mask[off] = static_cast<unsigned char>(s.m[pos_of(q)] | kDone);
+        st_rlx_u8(mask + off, s.m[pos_of(q)] | kDone);   // other tiles' visits read it meanwhile
       }
       out_any = __reduce_or_sync(kFull, out_any);
-      fence_ar();                               // the mask bytes before the activations
       __syncwarp();
+      fence_ar();                               // every lane's stores before the activations
       if ((out_any >> lane) & 1u) {                  // an upwind cell on face j lies in the grid
         const int ax = lane >> 1, d = (lane & 1) ? 1 : -1;
         const unsigned ux = tc[0] + (ax == 0 ? d : 0), uy = tc[1] + (ax == 1 ? d : 0), uz = tc[2] + (ax == 2 ? d : 0);
@@ -682,8 +686,8 @@ __global__ void __launch_bounds__(32, kAdjCtas) adj_tiles_kernel(const AdjProb *
       if (lane == 0) atomicAdd(&ctl->done, static_cast<unsigned long long>(ndone));
     }
     if (lane == 0) {
+      fence_ar();                               // and before the tile is another visit's
       finish_tile(sp, static_cast<unsigned long long>(tile));
-      fence_ar();
       atomicAdd(&sp.ctl->run[slot * kCounterPad], 0xffffffffu);
       atomicAdd(&sp.ctl->work, -1);
     }

@@ -59,10 +59,20 @@ def test_kernels_end_visits_that_way(name):
     assert not re.search(r"atomicCAS\(&\w+\.state", text)
 
 
-@pytest.mark.parametrize("name,call", [("eik_front.cu", "activate(p,"), ("eik_guided.cu", "activate(p,")])
+@pytest.mark.parametrize("name,call", [("eik_front.cu", "activate(p,"), ("eik_guided.cu", "activate(p,"),
+                                       ("eik_adjoint.cu", "        activate(sp,"),
+                                       ("eik_adjoint.cu", "finish_tile(sp,")])
 def test_fence_after_the_last_barrier(name, call):
     """Another lane's stores are covered only by a fence of the thread itself after
     the barrier between them."""
     text = frag.source(name)
     before = text[:text.index(call)]
     assert before.rfind("fence_ar();") > before.rfind("__syncwarp();")
+
+
+def test_adjoint_mask_bytes_are_stored_as_they_are_read():
+    """Visits of neighbouring tiles read the bytes while this one sets them: both
+    sides relaxed, neither plain."""
+    kernel = frag.block(frag.source("eik_adjoint.cu"), "adj_tiles_kernel(")
+    assert "ld_rlx_u8(mask" in kernel and "st_rlx_u8(mask" in kernel
+    assert not re.search(r"\bmask\[[^\]]*\]\s*[|&^]?=[^=]", kernel)
