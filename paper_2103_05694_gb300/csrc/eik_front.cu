@@ -59,6 +59,43 @@
 namespace eik {
 namespace {
 
+// The third warp's part of a visit: deliver the mail (lane j < 4: the bucket time of
+// face j) until the rounds are over (*fin) and no mail is left.  The rounds end
+// by themselves, after kMaxRounds at the latest, whatever timeout_ms is, so the
+// wait's own limit lies beyond that (a round takes about 1 us); lane 0 looks at the
+// clock for the whole warp, since the lanes' clocks differ and the votes need all of them.
+constexpr long long kVisitNs = 10ll * 1000 * 1000 * 1000;
+template <class Deliver>
+__device__ __forceinline__ void serve_mail(unsigned long long *mail, volatile int *fin, const SolveParams &p,
+                                           Deliver deliver) {
+  const int lane = threadIdx.x & 31;
+  const long long limit = p.timeout_ns > kVisitNs ? p.timeout_ns : kVisitNs;
+  long long t0 = 0;
+#pragma unroll 1
+  for (unsigned it = 0;; ++it) {
+    const bool over = *fin != 0;
+    __threadfence_block();
+    const unsigned long long m = lane < 4 ? atomicExch(&mail[lane], kEmpty) : kEmpty;
+    if (__any_sync(kFull, m != kEmpty)) {
+      deliver(m != kEmpty ? 1u << lane : 0u, m);
+      t0 = 0;
+      continue;
+    }
+    if (__all_sync(kFull, over)) break;
+    if ((it & 255u) == 255u) {
+      int late = 0;
+      if (lane == 0) {
+        const long long now = now_ns();
+        if (t0 == 0) t0 = now;
+        late = now - t0 > limit;
+        if (late) raise_status(p.ctl, kEtimeout, 8);
+      }
+      if (__shfl_sync(kFull, late, 0)) break;
+    }
+    __nanosleep(20);
+  }
+}
+
 // AHEAD, HELP (2D): see above.
 template <int D, bool AHEAD, bool HELP>
 __global__ void __launch_bounds__(HELP ? 96 : 64, HELP ? kFrontCtasHelp : D == 3 ? kFrontCtas3 : AHEAD ? kFrontCtas2 : kFrontCtasMany2)
@@ -191,24 +228,7 @@ __global__ void __launch_bounds__(HELP ? 96 : 64, HELP ? kFrontCtasHelp : D == 3
     if (HELP && warp == 2) {
 #pragma unroll 1
       for (;;) {
-        long long t0 = 0;
-#pragma unroll 1
-        for (unsigned it = 0;; ++it) {
-          const bool fin = sh_fin != 0;
-          __threadfence_block();
-          const unsigned long long m = lane < 4 ? atomicExch(&mail[lane], kEmpty) : kEmpty;
-          if (__any_sync(kFull, m != kEmpty)) {
-            activate_faces(m != kEmpty ? 1u << lane : 0u, m);
-            continue;
-          }
-          if (__all_sync(kFull, fin)) break;
-          if ((it & 255u) == 255u) {
-            const long long now = now_ns();
-            if (t0 == 0) t0 = now;
-            else if (now - t0 > p.timeout_ns) { if (lane == 0) raise_status(p.ctl, kEtimeout, 8); break; }
-          }
-          __nanosleep(20);
-        }
+        serve_mail(mail, &sh_fin, p, activate_faces);
         __syncwarp();
         if (lane == 0) {
           finish();
