@@ -295,7 +295,8 @@ eik_status eik_solve_noalloc(const double *speed, double h, int ndim, const int6
  *     shared memory; a tile is queued when a cell of it may have become ready;
  *   levels: one cooperative launch processes the cells level by level, its
  *     blocks meeting at a grid barrier between levels.
- * Every device wait is bounded by opts->timeout_ms (EIK_ETIMEOUT); opts->
+ * Every device wait is bounded by opts->timeout_ms (EIK_ETIMEOUT): a wait for
+ * work gives up when no cell has been processed anywhere for that long.  opts->
  * ctas_per_sm caps the CTAs of the tile schedule (0: chosen by the size of the
  * fronts).  Workspace: about 18 to 30 (tiles; 8 more for models
  * that problems share) or 53 (levels) bytes per cell of the batch, kept for the

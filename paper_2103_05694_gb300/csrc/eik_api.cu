@@ -2003,6 +2003,7 @@ extern "C" eik_status eik_adjoint(const eik_problem *probs, int nprob, const dou
       sp.cap_mask = (unsigned)(cap - 1);
       sp.ctl = adj().sched.p;
       sp.timeout_ns = tmo_ms * 1000000ll;
+      sp.progress = &adj().ctl.p->done;   // a call may take longer than timeout_ms, a standstill not
       sp.window = 31;
       CK(eik::launch_adjoint_tiles(adj().probs.p, nprob, total, total_tiles, hps[0].ndim, adj().ctl.p, sp,
                                    opts ? opts->ctas_per_sm : 0, opts && opts->counters, resume, s),

@@ -310,13 +310,16 @@ EIK_SCHED_FN unsigned long long take_slot(const SolveParams &p, unsigned s, unsi
 // `window` buckets of it are popped (bounded look-ahead, the soft priority of
 // OBIM).  On success the slot's run counter has been incremented for the
 // caller, `slot_out` is the slot and `lo_out` the lowest active bucket.
-// Returns kEmpty when the solve is over (done or error).
+// Returns kEmpty when the solve is over (done or error).  The wait gives up
+// timeout_ns after the last entry taken (idle_since), or, where the caller counts its
+// progress, when that count has stood still for so long.
 EIK_SCHED_FN unsigned long long pop_entry(const SolveParams &p, long long &idle_since,
                                         unsigned &slot_out, unsigned &lo_out) {
   Ctl *ctl = p.ctl;
   const unsigned lane = threadIdx.x & 31u;
   const unsigned win = p.window < 31u ? p.window : 31u;
   unsigned nap = 64;
+  unsigned long long seen = 0ull;       // *p.progress when idle_since was set
 #pragma unroll 1
   for (;;) {
     unsigned stop = 0, cur = 0;
@@ -389,8 +392,15 @@ EIK_SCHED_FN unsigned long long pop_entry(const SolveParams &p, long long &idle_
     }
     if (lane == 0) {
       const long long now = now_ns();
-      if (idle_since == 0) idle_since = now;
-      else if (now - idle_since > p.timeout_ns) raise_status(ctl, kEtimeout, 2);
+      if (idle_since == 0) {
+        idle_since = now;
+        if (p.progress) seen = ld_rlx(p.progress);
+      } else if (now - idle_since > p.timeout_ns) {
+        const unsigned long long got = p.progress ? ld_rlx(p.progress) : seen;
+        if (got == seen) raise_status(ctl, kEtimeout, 2);
+        seen = got;
+        idle_since = now;
+      }
     }
     // longer and longer: a scan is 66 L2 reads of lines that the working CTAs'
     // atomics need, and with many idle CTAs one looks soon anyway (at a fixed
