@@ -211,16 +211,45 @@ __global__ void adj_setup_kernel(const AdjProb *probs, int nprob, int64_t total,
   if ((threadIdx.x & 31) == 0 && reached) atomicAdd(&ctl->reached, reached);
 }
 
+// The cells of all problems, shared out for the set-up and the search for ready cells.
+// rows: a grid row per problem (first + blockIdx.y), so that no cell searches for
+// its problem.  Else one loop over all cells, which looks the problem up where it
+// changes: a row per problem gives each as many blocks as the average one needs, so
+// a batch whose largest problem is far above the average waits for that one (call
+// without the host's part, rows and one loop: a 256^3 volume beside 100 grids of
+// 20 x 21 x 22 27.9 and 8.8 ms, 3000^2 beside 200 of 40 x 50 26.1 and 9.5 to 11.2),
+// while like problems gain by the rows (3000 of 30 x 30, the same cells in equal
+// pieces of the loop: 0.53 and 0.57 ms, 2000 of 5 x 6 0.10 and 0.15).
+// cell(P, n) for each cell, leave(P) after a thread's last cell of P (rows: all
+// threads of a block together).
+template <class Cells, class Leave>
+__device__ __forceinline__ void for_cells(const AdjProb *probs, int nprob, int64_t total, int first, bool rows,
+                                          Cells cell, Leave leave) {
+  const int64_t at = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x,
+                step = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  if (rows) {
+    const AdjProb &P = probs[first + blockIdx.y];
+    const int64_t cells = P.nx * P.ny * P.nz;
+    for (int64_t n = at; n < cells; n += step) cell(P, n);
+    leave(P);
+    return;
+  }
+  for (int64_t q = at; q < total;) {
+    const AdjProb &P = probs[find_adj_prob(probs, nprob, q)];
+    const int64_t end = P.base + P.nx * P.ny * P.nz;
+    for (; q < end; q += step) cell(P, q - P.base);
+    leave(P);
+  }
+}
+
 // Tile schedule: the mask byte carries kPending (reached), and the problem's
-// largest time is collected (the tiles' order).  blockIdx.y: problem (first + y),
-// so that no cell searches for its problem and a warp needs one atomic.
-__global__ void adj_setup_tiles_kernel(const AdjProb *probs, int first, AdjCtl *ctl) {
-  const AdjProb &P = probs[first + blockIdx.y];
-  const int64_t total = P.nx * P.ny * P.nz;
+// largest time is collected (the tiles' order), with one atomic per warp where the
+// warp is of one problem; else only by those above what is there.
+template <bool ROWS>
+__global__ void adj_setup_tiles_kernel(const AdjProb *probs, int nprob, int64_t total, int first, AdjCtl *ctl) {
   unsigned long long reached = 0;
   unsigned top = 0u;        // high word of the largest finite time
-  for (int64_t n = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; n < total;
-       n += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+  for_cells(probs, nprob, total, first, ROWS, [&](const AdjProb &P, int64_t n) {
     const double tn = P.t[n];
     const bool is_reached = ubits(tn) < kInfB;
     if (is_reached) {
@@ -229,14 +258,18 @@ __global__ void adj_setup_tiles_kernel(const AdjProb *probs, int first, AdjCtl *
       top = top < hi ? hi : top;
     }
     P.mask[n] = static_cast<unsigned char>(setup_cell<false>(P, n, tn) | (is_reached ? kPending : 0u));
-  }
-  top = __reduce_max_sync(kFullMask, top);
+  }, [&](const AdjProb &P) {
+    if (ROWS) {
+      const unsigned m = __reduce_max_sync(kFullMask, top);
+      top = (threadIdx.x & 31) == 0 ? m : 0u;
+    }
+    const unsigned long long v = static_cast<unsigned long long>(top) << 32;
+    if (top && v > ld_rlx_u64(P.tmax)) atomicMax(P.tmax, v);
+    top = 0u;
+  });
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) reached += __shfl_xor_sync(kFullMask, reached, o);
-  if ((threadIdx.x & 31) == 0) {
-    if (reached) atomicAdd(&ctl->reached, reached);
-    if (top) atomicMax(P.tmax, static_cast<unsigned long long>(top) << 32);
-  }
+  if ((threadIdx.x & 31) == 0 && reached) atomicAdd(&ctl->reached, reached);
 }
 
 // Warp-aggregated append of the lanes' ready entries to a frontier.  All 32
@@ -430,28 +463,25 @@ __device__ __forceinline__ unsigned tile_bucket(const AdjProb &P, unsigned tx, u
 }
 
 // Queue the tiles holding a ready cell: reached, not done, and no neighbour that
-// is not done names its side.  blockIdx.y: problem (first + y).
-template <int TX, int TY, int TZ>
-__global__ void adj_tile_seed_kernel(const AdjProb *probs, int first, SolveParams sp) {
-  const AdjProb &P = probs[first + blockIdx.y];
-  const int64_t total = P.nx * P.ny * P.nz;
-  const unsigned char *const mask = P.mask;
-  const int64_t sy = P.nx, sz = P.nx * P.ny;
-  for (int64_t n = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; n < total;
-       n += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    if ((mask[n] & (kPending | kDone)) != kPending) continue;
+// is not done names its side.
+template <int TX, int TY, int TZ, bool ROWS>
+__global__ void adj_tile_seed_kernel(const AdjProb *probs, int nprob, int64_t total, int first, SolveParams sp) {
+  for_cells(probs, nprob, total, first, ROWS, [&](const AdjProb &P, int64_t n) {
+    const unsigned char *const mask = P.mask;
+    const int64_t sy = P.nx, sz = P.nx * P.ny;
+    if ((mask[n] & (kPending | kDone)) != kPending) return;
     const Cell e = cell_of(P, n);
     // neighbour at n + d waits for n, its side `side`
     auto uses = [&](int64_t d, int side) { return ((mask[n + d] >> side) & 1u) && !(mask[n + d] & kDone); };
     const bool used = (e.c[0] > 0 && uses(-1, 1)) || (e.c[0] + 1 < P.nx && uses(1, 0)) ||
                       (e.c[1] > 0 && uses(-sy, 3)) || (e.c[1] + 1 < P.ny && uses(sy, 2)) ||
                       (P.ndim == 3 && ((e.c[2] > 0 && uses(-sz, 5)) || (e.c[2] + 1 < P.nz && uses(sz, 4))));
-    if (used) continue;
+    if (used) return;
     const unsigned tx = static_cast<unsigned>(e.c[0] / TX), ty = static_cast<unsigned>(e.c[1] / TY),
                    tz = static_cast<unsigned>(e.c[2] / TZ);
     activate(sp, static_cast<unsigned long long>(P.tile_base) + (tz * P.nty + ty) * P.ntx + tx, 0u,
              tile_bucket<TX, TY, TZ>(P, tx, ty, tz));
-  }
+  }, [](const AdjProb &) {});
 }
 
 // TIMING: clocks of the visit phases and of the waits for work (the eik_stats
@@ -760,19 +790,30 @@ cudaError_t launch_adjoint(const AdjProb *probs_dev, int nprob, int64_t total, A
 namespace {
 
 template <int D, int TX, int TY, int TZ>
-cudaError_t run_tiles(const AdjProb *probs_dev, int nprob, int64_t total, int64_t total_tiles, AdjCtl *ctl,
-                      const SolveParams &sp, int ctas_per_sm, bool timing, bool resume, cudaStream_t stream) {
-  int64_t gx = (total / nprob + 255) / 256, share = (static_cast<int64_t>(sms()) * 8 + nprob - 1) / nprob;
-  if (gx > share) gx = share;
-  if (gx < 1) gx = 1;
-  for (int first = 0; first < nprob && !resume; first += 65535) {
-    const unsigned n = static_cast<unsigned>(nprob - first < 65535 ? nprob - first : 65535);
-    adj_setup_tiles_kernel<<<dim3(static_cast<unsigned>(gx), n), 256, 0, stream>>>(probs_dev, first, ctl);
-    note_launches(1);
-  }
-  for (int first = 0; first < nprob; first += 65535) {
-    const unsigned n = static_cast<unsigned>(nprob - first < 65535 ? nprob - first : 65535);
-    adj_tile_seed_kernel<TX, TY, TZ><<<dim3(static_cast<unsigned>(gx), n), 256, 0, stream>>>(probs_dev, first, sp);
+cudaError_t run_tiles(const AdjProb *probs_dev, int nprob, int64_t total, int64_t max_cells, int64_t total_tiles,
+                      AdjCtl *ctl, const SolveParams &sp, int ctas_per_sm, bool timing, bool resume, cudaStream_t stream) {
+  const int64_t all = static_cast<int64_t>(sms()) * 8, mean = total / nprob;
+  auto blocks_for = [](int64_t cells, int64_t most) {
+    const int64_t g = (cells + 255) / 256;
+    return static_cast<unsigned>(g < 1 ? 1 : g > most ? most : g);
+  };
+  if (max_cells <= 2 * mean) {
+    const unsigned gx = blocks_for(mean, (all + nprob - 1) / nprob);
+    for (int step = resume ? 1 : 0; step < 2; ++step) {
+      for (int first = 0; first < nprob; first += 65535) {
+        const dim3 grid(gx, static_cast<unsigned>(nprob - first < 65535 ? nprob - first : 65535));
+        if (step == 0) adj_setup_tiles_kernel<true><<<grid, 256, 0, stream>>>(probs_dev, nprob, total, first, ctl);
+        else adj_tile_seed_kernel<TX, TY, TZ, true><<<grid, 256, 0, stream>>>(probs_dev, nprob, total, first, sp);
+        note_launches(1);
+      }
+    }
+  } else {
+    const unsigned gx = blocks_for(total, all);
+    if (!resume) {
+      adj_setup_tiles_kernel<false><<<gx, 256, 0, stream>>>(probs_dev, nprob, total, 0, ctl);
+      note_launches(1);
+    }
+    adj_tile_seed_kernel<TX, TY, TZ, false><<<gx, 256, 0, stream>>>(probs_dev, nprob, total, 0, sp);
     note_launches(1);
   }
   // ctas_per_sm 0: what the fronts can use (a front of a problem of n tiles is
@@ -810,14 +851,14 @@ cudaError_t launch_adj_h2s(const double *v, int v_is_slowness, double hh, int64_
   return cudaGetLastError();
 }
 
-cudaError_t launch_adjoint_tiles(const AdjProb *probs_dev, int nprob, int64_t total, int64_t total_tiles,
-                                 int ndim, AdjCtl *ctl, const SolveParams &sp, int ctas_per_sm, bool timing,
-                                 bool resume, cudaStream_t stream) {
+cudaError_t launch_adjoint_tiles(const AdjProb *probs_dev, int nprob, int64_t total, int64_t max_cells,
+                                 int64_t total_tiles, int ndim, AdjCtl *ctl, const SolveParams &sp, int ctas_per_sm,
+                                 bool timing, bool resume, cudaStream_t stream) {
   if (ndim == 3)
-    return run_tiles<3, kAdjTile3[0], kAdjTile3[1], kAdjTile3[2]>(probs_dev, nprob, total, total_tiles, ctl, sp,
-                                                                  ctas_per_sm, timing, resume, stream);
-  return run_tiles<2, kAdjTile2[0], kAdjTile2[1], kAdjTile2[2]>(probs_dev, nprob, total, total_tiles, ctl, sp,
-                                                                ctas_per_sm, timing, resume, stream);
+    return run_tiles<3, kAdjTile3[0], kAdjTile3[1], kAdjTile3[2]>(probs_dev, nprob, total, max_cells, total_tiles, ctl,
+                                                                  sp, ctas_per_sm, timing, resume, stream);
+  return run_tiles<2, kAdjTile2[0], kAdjTile2[1], kAdjTile2[2]>(probs_dev, nprob, total, max_cells, total_tiles, ctl,
+                                                                sp, ctas_per_sm, timing, resume, stream);
 }
 
 }  // namespace eik

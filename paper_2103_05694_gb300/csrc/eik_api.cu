@@ -1862,10 +1862,11 @@ extern "C" eik_status eik_adjoint(const eik_problem *probs, int nprob, const dou
   }
   const bool tiles = adj_mode == 2 || (adj_mode == 0 && same_ndim && kAdjTilesDefault);
   const int *tsh = hps[0].ndim == 3 ? eik::kAdjTile3 : eik::kAdjTile2;
-  int64_t total_tiles = 0;
+  int64_t total_tiles = 0, max_cells = 0;
   std::vector<int64_t> ntile((size_t)nprob * 3);
   for (int i = 0; i < nprob; ++i) {
     const HostProblem &hp = hps[(size_t)i];
+    max_cells = std::max(max_cells, hp.n);
     const int64_t ext[3] = {hp.dims[2], hp.dims[1], hp.dims[0]};   // x, y, z
     for (int k = 0; k < 3; ++k) ntile[(size_t)i * 3 + k] = (ext[k] + tsh[k] - 1) / tsh[k];
     total_tiles += ntile[(size_t)i * 3] * ntile[(size_t)i * 3 + 1] * ntile[(size_t)i * 3 + 2];
@@ -2005,7 +2006,7 @@ extern "C" eik_status eik_adjoint(const eik_problem *probs, int nprob, const dou
       sp.timeout_ns = tmo_ms * 1000000ll;
       sp.progress = &adj().ctl.p->done;   // a call may take longer than timeout_ms, a standstill not
       sp.window = 31;
-      CK(eik::launch_adjoint_tiles(adj().probs.p, nprob, total, total_tiles, hps[0].ndim, adj().ctl.p, sp,
+      CK(eik::launch_adjoint_tiles(adj().probs.p, nprob, total, max_cells, total_tiles, hps[0].ndim, adj().ctl.p, sp,
                                    opts ? opts->ctas_per_sm : 0, opts && opts->counters, resume, s),
          "adjoint launch");
       CK(cudaMemcpyAsync(adj().sched_host, &adj().sched.p->status, sizeof(unsigned), cudaMemcpyDeviceToHost, s),

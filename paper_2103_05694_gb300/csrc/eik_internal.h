@@ -347,8 +347,9 @@ cudaError_t launch_adj_h2s(const double *v, int v_is_slowness, double hh, int64_
 constexpr int kAdjTile2[3] = {16, 16, 1};
 constexpr int kAdjTile3[3] = {8, 4, 4};
 constexpr int kAdjCtas = 12;
-cudaError_t launch_adjoint_tiles(const AdjProb *probs_dev, int nprob, int64_t total, int64_t total_tiles,
-                                 int ndim, AdjCtl *ctl, const SolveParams &sp, int ctas_per_sm, bool timing,
-                                 bool resume, cudaStream_t stream);
+// max_cells: of the largest problem.
+cudaError_t launch_adjoint_tiles(const AdjProb *probs_dev, int nprob, int64_t total, int64_t max_cells,
+                                 int64_t total_tiles, int ndim, AdjCtl *ctl, const SolveParams &sp, int ctas_per_sm,
+                                 bool timing, bool resume, cudaStream_t stream);
 
 }  // namespace eik
