@@ -782,8 +782,9 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
       all_t0.push_back(hp.t0[k]);
     }
   }
-  double t_min = lower ? ep->t_min : seeds.empty() ? 0.0 : seeds[0].t0;
-  for (const SeedItem &it : seeds) if (!lower) t_min = std::min(t_min, it.t0);
+  double t_first = seeds.empty() ? 0.0 : seeds[0].t0;      // the first source's time
+  for (const SeedItem &it : seeds) t_first = std::min(t_first, it.t0);
+  const double t_min = lower ? ep->t_min : t_first;        // the first that sends out a front
   if (total_tiles >= (int64_t(1) << 32)) { set_err("too many tiles"); return EIK_EINVAL; }
   CK(ws().state.ensure((size_t)total_tiles), "alloc tile state");
   CK(ws().tile_src.ensure((size_t)total_tiles), "alloc tile flags");
@@ -934,7 +935,7 @@ eik_status run(std::vector<HostProblem> &hps, const eik_opts *opts, eik_stats *s
     CK(clear_scheduler(ws().ctl.p, stream), "clear scheduler");
     CK(cudaMemsetAsync(ws().state.p, 0, (size_t)total_tiles * sizeof(unsigned long long), stream),
        "clear tile states");
-    CK(eik::launch_reseed(sp, probs.data(), (int)probs.size(), stream), "reseed launch");
+    CK(eik::launch_reseed(sp, probs.data(), (int)probs.size(), stream, t_first), "reseed launch");
     acc.retries++;
   }
   if (status != 0) {
@@ -1517,7 +1518,7 @@ struct eik_plan {
   Ctl *ctl_host = nullptr;
   SolveParams sp;
   int grid = 1;
-  double k_delta = 0.0, delta_fixed = 0.0;
+  double k_delta = 0.0, delta_fixed = 0.0, t_min = 0.0;   // t_min: of the sources
   int from_slowness = 0;
   uint64_t cap = 0;
 
@@ -1644,6 +1645,8 @@ eik_status plan_build(eik_plan &pl, std::vector<HostProblem> &hps, const eik_opt
     }
   }
   pl.nseeds = (int64_t)seeds.size();
+  pl.t_min = seeds.empty() ? 0.0 : seeds[0].t0;
+  for (const SeedItem &it : seeds) pl.t_min = std::min(pl.t_min, it.t0);
   if (pl.total_tiles >= (int64_t(1) << 32)) { set_err("too many tiles"); return EIK_EINVAL; }
   CK(pl.state.ensure((size_t)pl.total_tiles), "plan: alloc tile state");
   CK(pl.tile_src.ensure((size_t)pl.total_tiles), "plan: alloc tile flags");
@@ -1768,7 +1771,7 @@ eik_status eik_plan_enqueue(eik_plan *pl, void *stream) {
                           pl->ctl.p, s, pl->sp.update != 0, pl->from_slowness), "init_c launch");
   }
   CK(eik::launch_init_t_all(pl->sp.probs, (int)pl->probs.size(), pl->max_cells, s), "init_t launch");
-  CK(eik::launch_seed(pl->sp, pl->seeds.p, pl->nseeds, pl->k_delta, pl->delta_fixed, s), "seed launch");
+  CK(eik::launch_seed(pl->sp, pl->seeds.p, pl->nseeds, pl->k_delta, pl->delta_fixed, s, pl->t_min), "seed launch");
   CK(eik::launch_persistent(pl->sp, pl->grid, s), "solve launch");
   if (pl->ncopies)
     CK(eik::launch_copy_items(pl->copies.p, pl->ncopies, pl->copy_max_n, s), "plan: copy launch");

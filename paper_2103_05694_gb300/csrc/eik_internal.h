@@ -219,7 +219,7 @@ cudaError_t launch_seed(const SolveParams &p, const SeedItem *items, int64_t nit
                         double k_delta, double delta_fixed, cudaStream_t stream, double t_min = 0.0,
                         bool lower = false);
 cudaError_t launch_reseed(const SolveParams &p, const Prob *host_probs, int nprob,
-                          cudaStream_t stream);
+                          cudaStream_t stream, double t_min = 0.0);
 cudaError_t launch_persistent(const SolveParams &p, int grid, cudaStream_t stream);
 // The guided and the front kernel (tile_shape kGuidedShape0 and kFrontShape).
 cudaError_t launch_guided(const SolveParams &p, int grid, cudaStream_t stream);

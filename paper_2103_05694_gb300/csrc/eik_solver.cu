@@ -755,9 +755,11 @@ __global__ void seed_kernel(SolveParams p, const SeedItem *__restrict__ items, i
 }
 
 // Capacity retry: every tile holding a finite value is re-queued with a full
-// evaluation (Theorem 1: any state reached by valid updates is a valid start).
-__global__ void reseed_kernel(SolveParams p, int tx_, int ty_, int tz_, int64_t total_tiles) {
+// evaluation (Theorem 1: any state reached by valid updates is a valid start).  The
+// scheduler's hint starts at t_min's bucket, as in seed_kernel.
+__global__ void reseed_kernel(SolveParams p, int tx_, int ty_, int tz_, int64_t total_tiles, double t_min) {
   const float inv = static_cast<float>(p.ctl->inv_delta);
+  const unsigned base = bucket_of_time(bits_of(t_min), inv);
   for (int64_t g = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; g < total_tiles;
        g += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const int pi = find_prob(p, static_cast<unsigned long long>(g));
@@ -777,7 +779,7 @@ __global__ void reseed_kernel(SolveParams p, int tx_, int ty_, int tz_, int64_t 
         for (int64_t x = x0; x < x1; ++x)
           best = umin64(best, bits_of(ld_time(P.t + (z * P.ny + y) * P.nx + x)));
     if (best < kInfBits) activate(p, static_cast<unsigned long long>(g), 1u << kFaceFull,
-                                  bucket_of_time(best, inv));
+                                  bucket_of_time(best, inv), base);
   }
 }
 
@@ -978,13 +980,17 @@ static void tile_dims(const SolveParams &p, int &tx, int &ty, int &tz) {
   tz = ts.tz;
 }
 
+// The lowest-bucket hint before items of which none is earlier than t_min are pushed:
+// the pushes lower it to the smallest bucket.
+static cudaError_t start_hint(const SolveParams &p, double t_min, cudaStream_t stream) {
+  return t_min > 0.0 ? cudaMemsetAsync(&p.ctl->cur, 0xff, sizeof(p.ctl->cur), stream) : cudaSuccess;
+}
+
 cudaError_t launch_seed(const SolveParams &p, const SeedItem *items, int64_t nitems,
                         double k_delta, double delta_fixed, cudaStream_t stream, double t_min,
                         bool lower) {
-  if (t_min > 0.0) {   // the pushes below lower the hint to the smallest bucket
-    const cudaError_t e = cudaMemsetAsync(&p.ctl->cur, 0xff, sizeof(p.ctl->cur), stream);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = start_hint(p, t_min, stream);
+  if (e != cudaSuccess) return e;
   int tx, ty, tz;
   tile_dims(p, tx, ty, tz);
   const int grid = grid_for(nitems > 0 ? nitems : 1, 4);
@@ -994,12 +1000,14 @@ cudaError_t launch_seed(const SolveParams &p, const SeedItem *items, int64_t nit
 }
 
 cudaError_t launch_reseed(const SolveParams &p, const Prob *host_probs, int nprob,
-                          cudaStream_t stream) {
+                          cudaStream_t stream, double t_min) {
+  const cudaError_t e = start_hint(p, t_min, stream);
+  if (e != cudaSuccess) return e;
   int tx, ty, tz;
   tile_dims(p, tx, ty, tz);
   const Prob &last = host_probs[nprob - 1];
   const int64_t total = last.tile_base + last.ntx * last.nty * last.ntz;
-  reseed_kernel<<<grid_for(total, 4), 256, 0, stream>>>(p, tx, ty, tz, total);
+  reseed_kernel<<<grid_for(total, 4), 256, 0, stream>>>(p, tx, ty, tz, total, t_min);
   note_launches(1);
   return cudaGetLastError();
 }
