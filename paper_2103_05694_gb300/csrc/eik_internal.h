@@ -53,7 +53,9 @@ struct Ctl {
   double inv_delta;
   unsigned long long rmin_bits;   // smallest r (bit pattern; all r > 0)
   int scale_exp;            // binary exponent of the mean r (the guided kernel's float unit)
-  int pad3[21];
+  int pad3;
+  double t_first;           // the first source's time, where only the device knows it (else 0)
+  int pad4[18];
   unsigned long long stats[kNumStats];
   unsigned long long error_info[4];   // where a wait gave up / what was invalid
   unsigned long long trace_n;         // trace records written (may exceed the capacity)

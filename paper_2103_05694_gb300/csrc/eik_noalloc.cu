@@ -119,13 +119,19 @@ sources_kernel(const int64_t *__restrict__ src_idx, const double *__restrict__ s
   }
   if (tid == 0) {   // compaction (n <= 2048, once per call)
     int u = 0;
+    unsigned long long first = ~0ull;            // bits of the smallest time
     for (int i = 0; i < n; ++i) {
       if (i > 0 && key_idx[i] == key_idx[i - 1]) continue;
       out_idx[u] = static_cast<int64_t>(key_idx[i]);
       out_t[u] = __longlong_as_double(static_cast<long long>(key_t[i]));
+      first = first < key_t[i] ? first : key_t[i];
       ++u;
     }
     s_nuniq = u;
+    if (u > 0 && first > 0ull) {                 // the seeds' pushes lower the hint to its bucket
+      ctl->t_first = __longlong_as_double(static_cast<long long>(first));
+      ctl->cur = ~0u;
+    }
     prob.src_idx = out_idx;
     prob.src_t = out_t;
     prob.nsrc = u;

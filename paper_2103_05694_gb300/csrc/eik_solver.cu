@@ -719,7 +719,7 @@ __global__ void seed_kernel(SolveParams p, const SeedItem *__restrict__ items, i
                                    : k_delta * (ctl->rsum / static_cast<double>(ctl->rcount));
   if (!(delta > 0.0) || !(bits_of(delta) < kInfBits)) delta = 1.0;
   const double inv = 1.0 / delta;
-  const unsigned base = bucket_of_time(bits_of(t_min), static_cast<float>(inv));
+  const unsigned base = bucket_of_time(bits_of(t_min > 0.0 ? t_min : ctl->t_first), static_cast<float>(inv));
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl->delta = delta;
     ctl->inv_delta = inv;

@@ -1,5 +1,5 @@
-"""Source times far from 0: plans, and solves that go on after a bucket slot
-overflowed, start at the first source's bucket like a plain solve.  From bucket 0
+"""Source times far from 0: plans, the solve without allocation and solves that go
+on after a bucket slot overflowed start at the first source's bucket like a plain solve.  From bucket 0
 every tile would be clamped to the ring's last slot, in no order, which shows in
 the number of visits; the bits are the oracle's either way."""
 import numpy as np
@@ -69,4 +69,20 @@ def test_resumed_solve(shape):
         assert r.stats["retries"] > 0
         visits.append(r.stats["visits"])
     assert np.array_equal(_bits(r.t.cpu().numpy()), _bits(oracle.fmm(speed, 0.5, src, times).t))
+    assert visits[1] < 2 * visits[0]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_noalloc(shape):
+    visits = []
+    for t0 in (0.0, T0):
+        speed, src, times = _problem(shape, t0)
+        dev = [torch.from_numpy(x).to(DEV) for x in (speed, src, times)]
+        out = torch.full_like(dev[0], -1.0)
+        stats = eik.eik_solve_noalloc(dev[0].data_ptr(), 0.5, speed.ndim, speed.shape, dev[1].data_ptr(),
+                                      dev[2].data_ptr(), src.size, out.data_ptr(), {"counters": 1},
+                                      torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        visits.append(stats["visits"])
+    assert np.array_equal(_bits(out.cpu().numpy()), _bits(oracle.fmm(speed, 0.5, src, times).t))
     assert visits[1] < 2 * visits[0]
