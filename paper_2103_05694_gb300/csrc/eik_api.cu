@@ -1652,9 +1652,14 @@ eik_status plan_build(eik_plan &pl, std::vector<HostProblem> &hps, const eik_opt
   CK(pl.tile_src.ensure((size_t)pl.total_tiles), "plan: alloc tile flags");
   if (!use_guided(opts))
     CK(pl.pend.ensure((size_t)pl.total_tiles * eik::kPendWords), "plan: alloc pending masks");
-  uint64_t want_cap = opts && opts->capacity > 0 ? (uint64_t)opts->capacity
-                                                 : (uint64_t)pl.total_tiles / 2 + 4096;
-  if (use_guided(opts)) want_cap = std::max<uint64_t>(want_cap, (uint64_t)pl.total_tiles / 2 + 4096);
+  // A plan cannot grow its ring.  In 2D the front kernel has twice as many tiles as
+  // the other kernel with many fronts, so what filled half of a slot there fills
+  // all of it here: twice the other kernel's room, where there are so many tiles.
+  const uint64_t nt = (uint64_t)pl.total_tiles;
+  const uint64_t auto_cap =
+      shape == eik::kFrontShape && pl.ndim == 2 ? std::max(nt / 2 + 4096, std::min(nt, nt / 2 + 8192)) : nt / 2 + 4096;
+  uint64_t want_cap = opts && opts->capacity > 0 ? (uint64_t)opts->capacity : auto_cap;
+  if (use_guided(opts)) want_cap = std::max<uint64_t>(want_cap, auto_cap);
   want_cap = next_pow2(std::max<uint64_t>(want_cap, 16));
   while (want_cap * eik::kNumSlots > kMaxCapEntries && want_cap > 1024) want_cap >>= 1;
   pl.cap = want_cap;
