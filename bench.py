@@ -435,14 +435,14 @@ def roofline(useful_per_launch: int, kern_ms: float, traffic, what: str):
             "peak_kind": f"{kind} copy bandwidth"}
 
 
-def roofline_fp64(C, evals_per_launch: int, kern_ms: float, ndim: int, what: str,
+def roofline_fp64(C, evals_per_launch: int | None, kern_ms: float, ndim: int, what: str,
                   workload: str | None = None):
     """The FP64 roofline of the tile kernel: FP64 thread instructions per
     launch (ncu instructions per evaluation x the live evaluation count) over the
     kernel's event time, against the device's measured FP64 add rate."""
     per_eval = MEASURED_FP64_PER_EVAL.get(workload, MEASURED_FP64_PER_EVAL.get(ndim))
     peak = C.eik.eik_fp64_rate() / 1e9
-    if per_eval is None:
+    if per_eval is None or evals_per_launch is None:   # None: the timed kernel does not count
         return {"bound": "fp64", "achieved": None, "peak": peak, "unit": "G FP64 inst/s",
                 "frac": None, "kernel": what, "note": "FP64 instructions per evaluation not "
                 "measured for this build", "peak_kind": "measured (eik_fp64_rate, DADD chains)"}
@@ -451,6 +451,32 @@ def roofline_fp64(C, evals_per_launch: int, kern_ms: float, ndim: int, what: str
             "frac": achieved / peak, "kernel": what, "kernel_ms": kern_ms,
             "fp64_inst_per_eval": per_eval, "evals_per_launch": int(evals_per_launch),
             "peak_kind": "measured (eik_fp64_rate, DADD chains)"}
+
+
+def counting_kernel_runs(opts: dict) -> bool:
+    """Whether a solve with these options runs the kernel that can count its work.
+    With automatic scheduling options (or arith 3) the front or guided kernel runs,
+    which has no counters: a solve with counters=1 is another kernel's launch."""
+    if opts.get("update") or opts.get("schedule") or opts.get("sched_flags", 0) & (1 | 6 | 32):
+        return True
+    if opts.get("arith", 0) == 3:
+        return False
+    return bool(opts.get("arith", 0)) or any(
+        opts.get(k, 0) > 0 for k in ("delta", "k_delta", "window", "band", "ctas_per_sm", "tile"))
+
+
+WORK_FIELDS = ("evals", "decreases", "good", "visits", "pushes", "stale_pops", "rounds")
+
+
+def work_per_step(st: dict, opts: dict) -> dict:
+    """The work of one timed step, from the statistics of a counting solve with the
+    same options.  "good" (cells that got a value) does not depend on the kernel;
+    the rest is null where the timed kernel does not count."""
+    if counting_kernel_runs(opts):
+        return dict({k: st[k] for k in WORK_FIELDS}, empty=st["evals"] - st["decreases"],
+                    bad=st["decreases"] - st["good"])
+    return dict({k: None for k in WORK_FIELDS + ("empty", "bad")}, good=st["good"],
+                note="the timed kernel has no counters")
 
 
 def base_line(args, n, wl_name, value, total_ms, extra_cfg):
@@ -557,11 +583,9 @@ def run_single(args, C, wl_name):
     line = base_line(args, n, wl_name, value, total_ms,
                      {"cells": prob.ncells, "h": prob.h, "sources": int(len(prob.sources)),
                       "opts": opts, "autotune": tune})
-    line["grid_point_updates_per_s"] = st["evals"] * args.steps * n / (total_ms / 1e3)
-    line["work_per_step"] = {k: st[k] for k in ("evals", "decreases", "good", "visits", "pushes",
-                                                "stale_pops", "rounds")}
-    line["work_per_step"].update(empty=st["evals"] - st["decreases"],
-                                 bad=st["decreases"] - st["good"])
+    line["work_per_step"] = work_per_step(st, opts)
+    evals = line["work_per_step"]["evals"]
+    line["grid_point_updates_per_s"] = None if evals is None else evals * args.steps * n / (total_ms / 1e3)
     line["residual"] = {"update": ["d-bar", "d-tilde", "d-hat", "d-hat+Newton"][args.update]
                         + (" (change tracking)" if args.track_changes else ""), "cells": bad,
                         "max_rel": max_rel, "same_bits_every_step": same_bits}
@@ -574,7 +598,7 @@ def run_single(args, C, wl_name):
                                  "topo_kernel (Algorithm 4 iterations)",
                                  "fsm_kernel (Algorithm 5 sweeps)"][args.schedule])
     if args.schedule == 0:
-        line["roofline_fp64"] = roofline_fp64(C, st["evals"], statistics.mean(solve_ms),
+        line["roofline_fp64"] = roofline_fp64(C, evals, statistics.mean(solve_ms),
                                               prob.speed.ndim, line["roofline"]["kernel"],
                                               args.workload)
     line["e2e"] = {"value": useful * n / (e2e_ms / 1e3), "unit": UNIT, "ms_per_step": e2e_ms,
@@ -679,15 +703,12 @@ def run_batched(args, C, wl_name):
     if n > 1:
         line["scaling"] = "strong"
         line["config"]["parallelism"] = f"sharded by problem x{n} (rank r: problems r, r+{n}, ...)"
-    line["work_per_step"] = {k: st[k] for k in ("evals", "decreases", "good", "visits", "pushes",
-                                                "stale_pops", "rounds")}
-    line["work_per_step"].update(empty=st["evals"] - st["decreases"],
-                                 bad=st["decreases"] - st["good"])
+    line["work_per_step"] = work_per_step(st, opts)
     line["roofline"] = roofline(useful_mine, statistics.mean(solve_ms), args.traffic_bytes,
                                 "tile kernel (all problems in one launch)")
     if args.problems == 0:
         line["roofline"]["traffic_default_options"] = BATCH_TRAFFIC_DEFAULT_OPTIONS
-    line["roofline_fp64"] = roofline_fp64(C, st["evals"], statistics.mean(solve_ms), 3,
+    line["roofline_fp64"] = roofline_fp64(C, line["work_per_step"]["evals"], statistics.mean(solve_ms), 3,
                                           line["roofline"]["kernel"], "batched_3d")
     line["e2e"] = {"value": useful_all / (e2e_ms / 1e3), "unit": UNIT, "ms_per_step": e2e_ms,
                    "h2d_bytes_per_step": int(h2d), "d2h_bytes_per_step": int(d2h),
@@ -787,7 +808,6 @@ def run_tomography(args, C, wl_name):
 
     # kernel-only duration of the batched forward launch
     probs = [{"speed": s0, "h": h, "sources": src, "out": outs[i]} for i, src in enumerate(srcs)]
-    fwd_evals = eik.eik_solve_batched(probs, {"sched_flags": eik.SLOWNESS_INPUT, "counters": 1})["evals"]
     solve_ms = [eik.eik_solve_batched(probs, {"sched_flags": eik.SLOWNESS_INPUT})["solve_ms"]
                 for _ in range(3)]
 
@@ -816,7 +836,7 @@ def run_tomography(args, C, wl_name):
                                                     if per_source_ms else None)}
     line["roofline"] = roofline(len(srcs) * (s0.numel() - 1), statistics.mean(solve_ms),
                                 args.traffic_bytes, "tile kernel (batched forward)")
-    line["roofline_fp64"] = roofline_fp64(C, fwd_evals, statistics.mean(solve_ms), 2,
+    line["roofline_fp64"] = roofline_fp64(C, None, statistics.mean(solve_ms), 2,
                                           line["roofline"]["kernel"])
     line["e2e"] = {"value": useful_all / (e2e_ms / 1e3), "unit": UNIT, "ms_per_step": e2e_ms,
                    "h2d_bytes_per_step": int(h_s.numel() * 8),
