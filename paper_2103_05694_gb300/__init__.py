@@ -163,7 +163,7 @@ EXPORTED = ["eik_solve", "eik_solve_batched", "eik_release", "eik_status_str", "
             "eik_sum_ordered", "eik_solve_slabs", "eik_fp64_rate"]
 
 SELFTEST_CHECKS = ["sub", "sq", "add", "G2", "G3", "dbar2", "dbar3", "group2x8", "group3x8",
-                   "group2x4", "dbar2_fp64", "dbar3_fp64"]
+                   "group2x4", "dbar2_fp64", "dbar3_fp64", "quotient", "dbar2_kept", "dbar3_kept"]
 
 
 def eik_selftest(n: int = 1 << 20, seed: int = 1, stream=None) -> dict:

@@ -2,8 +2,9 @@
 // hardware FP64 unit, bit for bit, on random and tie-heavy inputs generated on
 // the device from a counter-based hash (splitmix64 of seed and index).
 //
-// Checked: fl(x - y), fl(m * m), fl(x + y), G(tau) in 2D and 3D, and d-bar in
-// 2D and 3D, where the reference d-bar is the plain definition: bisection over
+// Checked: fl(x - y), fl(m * m), fl(x + y), fl(x / y), G(tau) in 2D and 3D, and
+// d-bar in 2D and 3D (also with the constants of a cell kept from one evaluation to
+// the next), where the reference d-bar is the plain definition: bisection over
 // bit patterns for the smallest tau with G_hw(tau) >= c, G_hw built from
 // __dsub_rn / __dmul_rn / __dadd_rn.
 #include <cstdint>
@@ -95,9 +96,44 @@ __device__ bool group_ok(const unsigned long long (&a_in)[D], unsigned long long
   return dec == want && (!dec || out == ref);
 }
 
+// d-bar of a cell whose minima fall, into lower binades too, with one Scaled for all
+// evaluations.
+template <int D>
+__device__ bool kept_ok(const unsigned long long (&a_in)[D], unsigned long long cb) {
+  ig::Scaled<D> kept;
+  unsigned long long a[D];
+  bool ok = true;
+#pragma unroll 1
+  for (int rep = 0; rep < 4; ++rep) {
+#pragma unroll
+    for (int k = 0; k < D; ++k)
+      a[k] = a_in[k] >= kInf ? kInf : as_u(__dmul_rn(as_d(a_in[k]), 1.0 - 0.25 * rep));
+    ok = ok && hw::dbar<D>(a, cb, nullptr, kept) == dbar_ref<D>(a, cb);
+  }
+  return ok;
+}
+
+// A divisor or dividend: exponents anywhere, or at the ends of the integer form's
+// range, or subnormal; significands random, few bits, all ones.
+__device__ unsigned long long quotient_arg(unsigned long long h) {
+  const int pick = static_cast<int>((h >> 52) & 15u);
+  int e = 923 + static_cast<int>((h >> 56) % 200u);
+  if (pick == 0) e = 62 + static_cast<int>((h >> 56) % 4u);
+  if (pick == 1) e = 1998 + static_cast<int>((h >> 56) % 5u);
+  if (pick == 2) e = static_cast<int>((h >> 56) % 3u);
+  if (pick == 3) e = 2046 - static_cast<int>((h >> 56) % 3u);
+  unsigned long long m = mix(h) & xf::kFrac;
+  const unsigned sel = static_cast<unsigned>(h & 7u);
+  if (sel == 0) m = 0ull;
+  if (sel == 1) m = xf::kFrac - (m & 3ull);
+  if (sel == 2) m &= 3ull;
+  return (static_cast<unsigned long long>(e) << 52) | m;
+}
+
 // counters: 0 sub, 1 sq, 2 add, 3 G2, 4 G3, 5 dbar2, 6 dbar3, 7 group 2D x8,
-// 8 group 3D x8, 9 group 2D x4, 10 FP64-unit dbar 2D, 11 3D; [15] trials;
-// [16 + k] first failing trial of check k
+// 8 group 3D x8, 9 group 2D x4, 10 default dbar 2D, 11 3D, 12 quotient, 13 default
+// dbar with kept constants 2D, 14 3D; [15] trials; [16 + k] first failing trial of
+// check k
 __global__ void selftest_kernel(int64_t n, unsigned long long seed, unsigned long long *bad,
                                 unsigned long long *first) {
   // whole warps iterate together (the lane-group checks use warp collectives)
@@ -107,7 +143,7 @@ __global__ void selftest_kernel(int64_t n, unsigned long long seed, unsigned lon
     const bool live = i < n;
     const unsigned long long h0 = mix(seed ^ mix(static_cast<unsigned long long>(i)));
     const unsigned long long h1 = mix(h0), h2 = mix(h1), h3 = mix(h2), h4 = mix(h3), h5 = mix(h4);
-    unsigned long long nb[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+    unsigned long long nb[15] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     // sub and add: x >= y > 0 with exponent gaps 0..70
     {
       unsigned long long x = rand_double(h1, 900, 250);
@@ -154,8 +190,18 @@ __global__ void selftest_kernel(int64_t n, unsigned long long seed, unsigned lon
       if (!group_ok<2, 8>(a2, cb, hg)) nb[7] = 1;
       if (!group_ok<3, 8>(a3, cb, hg)) nb[8] = 1;
       if (!group_ok<2, 4>(a2, cb, hg ^ 1)) nb[9] = 1;
+      if (!kept_ok<2>(a2, cb)) nb[13] = 1;
+      if (!kept_ok<3>(a3, cb)) nb[14] = 1;
     }
-    for (int k = 0; k < 12; ++k) {
+    {
+      unsigned long long x = quotient_arg(mix(h0 ^ 5));
+      if (x == 0ull) x = 1ull;                                                 // positive
+      unsigned long long y = quotient_arg(mix(h0 ^ 6));
+      if ((h0 & 0xff00ull) == 0ull) y = (h0 & 1ull) ? kInf : (y | (1ull << 63));
+      const double q = ig::quotient(as_d(x), as_d(y)), want = __ddiv_rn(as_d(x), as_d(y));
+      if (as_u(q) != as_u(want)) nb[12] = 1;
+    }
+    for (int k = 0; k < 15; ++k) {
       if (live && nb[k]) {
         atomicAdd(&bad[k], 1ull);
         atomicCAS(&first[k], ~0ull, static_cast<unsigned long long>(i));

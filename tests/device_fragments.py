@@ -27,5 +27,5 @@ def block(text: str, head: str) -> str:
 def run(tmp_path, program: str, *args) -> subprocess.CompletedProcess:
     src, exe = tmp_path / "fragment.cpp", tmp_path / "fragment"
     src.write_text(program)
-    subprocess.run(["g++", "-std=c++17", "-O1", "-pthread", "-w", "-o", str(exe), str(src)], check=True, timeout=300)
+    subprocess.run(["g++", "-std=c++17", "-O2", "-ffp-contract=off", "-pthread", "-w", "-o", str(exe), str(src)], check=True, timeout=300)
     return subprocess.run([str(exe), *map(str, args)], capture_output=True, text=True, timeout=300)
