@@ -31,7 +31,7 @@
 // 1024^2 13262 -> 11214; a layered section takes about 1950 cycles per cell of its
 // longest chain.  It evaluates a cell more often (28 times on the section), so
 // where there are fronts enough to fill the device with ordered work the guided
-// kernel stays ahead (88-problem 3D batch: 57 against 135 ms).
+// kernel stays ahead (88-problem 3D batch: 43 against 78 ms).
 // One warp of two cells per lane: 5290 against 4086 us on the section (1.7
 // evaluations per round), but 7.6 against 8.0 ms on the checkerboard.
 // In 2D, where CTAs are free for it (SolveParams::ahead), a tile that a first front

@@ -116,7 +116,8 @@ struct SolveParams {
   unsigned long long trace_cap;
   int wide;                       // lean launches of 4x4x4 3D tiles: the build compiled for
                                   // EIK_WIDE_CTAS_64 CTAs per SM (fewer registers)
-  int guided;                     // 1: the guided kernel (eik_guided.cu; lean solves only)
+  int guided;                     // 1: the kernel that tile_shape names, front or guided (lean
+                                  // solves with automatic options)
 };
 
 // One tile visit, for timeline analysis (opts.trace).

@@ -1,5 +1,5 @@
 // Device helpers and the bucket scheduler shared by the tile kernels
-// (eik_solver.cu, eik_guided.cu): bit-pattern arithmetic, relaxed and
+// (eik_solver.cu, eik_front.cu, eik_guided.cu, eik_adjoint.cu): bit-pattern arithmetic, relaxed and
 // acquire/release accesses, and the ring of bucket slots (push, pop, claim,
 // finish).
 #pragma once
@@ -403,9 +403,9 @@ EIK_SCHED_FN unsigned long long pop_entry(const SolveParams &p, long long &idle_
       }
     }
     // longer and longer: a scan is 66 L2 reads of lines that the working CTAs'
-    // atomics need, and with many idle CTAs one looks soon anyway (at a fixed
-    // 128 ns a 600 x 500 adjoint takes 2.31 ms, 24 sections 1.92, with this 2.04
-    // and 1.75)
+    // atomics need, and with many idle CTAs one looks soon anyway (24 sections of
+    // 150 to 400 by 300 to 800 cells: 2.87 ms at a fixed 128 ns, 2.65 with this;
+    // adjoints of one to four 600 x 500 fields, with CTAs by their size: the same)
     __nanosleep(nap);
     nap = nap < 4096u ? 2u * nap : 4096u;
   }
