@@ -402,9 +402,10 @@ __global__ void __launch_bounds__(kThreads) adj_levels_kernel(const AdjProb *pro
 // the cell in the tile's middle, in fractions of the problem's largest time), so
 // that a tile's users are mostly done when it is taken.
 //
-// What bounds it: the chain of tiles (a visit is about 40 kcycles, of which the
-// loads and the stores take three quarters), so many small tiles in flight count,
-// and few visits per tile.  Against per-cell counts (two arrays, atomics in the
+// What bounds it: the chain of tiles.  A visit is 56 kcycles in 2D (32 problems of
+// 1024^2 cells: loads 18, 21 rounds 26, stores and hand-over 13; 1.6 visits per tile)
+// and 33 in 3D (8 of 90 x 101 x 110: 11, 10 and 12; 3.1 visits), at 4 to 16 % of the
+// issue slots, so many small tiles in flight count, and few visits per tile.  Against per-cell counts (two arrays, atomics in the
 // set-up and at every release), a FIFO of tiles and a block of 128 (2D) or 256
 // threads per tile with a barrier per round: 8.97 -> 4.97 ms for 32 problems of
 // 1024^2 cells, 6.6 -> 3.6 ms for one of 192 x 224 x 208.  Tiles: 16x16 in 2D
