@@ -397,13 +397,17 @@ bool use_guided(const eik_opts *o) {
 // automatic options.  The front kernel wherever the length of the fronts bounds the
 // solve; with many fronts in a large volume there is ordered work for every warp,
 // and the guided kernel's fewer evaluations win (batches of 128^3 grids, front
-// against guided: 16.8 M cells 5.7 and 8.7 ms, 33.5 M 10.5 and 11.3, 67 M 20.8 and
-// 16.5, 185 M 58 and 36).  CTAs per SM: a single 2D front has few active tiles, and
+// against guided: 16.8 M cells 6.2 and 8.2 ms, 33.5 M 12.7 and 11.7, 67 M 25.8 and
+// 17.8, 185 M 72 and 41; one grid of 46.7 M cells 21.1 ms with 1 source, 21.5 with 7,
+// and on the guided side 18.5 with 8 spread ones, 19.3 with a cluster of 27, 23.8 with a
+// line of 360; other kernel 34.0, 36.4 and 48.9).  CTAs per SM: a single 2D front has few active tiles, and
 // more CTAs take tiles out of order (751 x 2301 section: 3 to 5 CTAs 3.3 ms, 6 3.2,
 // 8 3.5; 1502 x 4602: 9.5, 8.1, 7.6, 7.4 and 7.4 ms); elsewhere as many as fit (24
 // sections: 8 CTAs 1.66 ms, 10 1.55, 12 1.52, 16 with spills more; 256^3 checkerboard: 8 10.9 ms, 12 8.7,
-// 14 8.0, 20 with spills 9.3; 97 x 131 x 203: 12 1.76, 14 1.82, 16 2.1; many 3D
-// fronts launch the 20 of the other kernels, of which 14 run at a time).  Bucket
+// 14 8.0, 20 with spills 9.3; 97 x 131 x 203: 12 1.76, 14 1.82, 16 2.1).  Many 3D
+// fronts launch 20, the number reported for both kernels that run them; 14 of the
+// front kernel's fit, and the others start when the work is over (8 problems of 128^3
+// 6.23 ms, launching 14 6.22; 20 uneven grids 1.49 and 1.48).  Bucket
 // widths: the layered section 4.4 ms at 8, 4.2 at 16, 4.1 at 32 (before the look
 // ahead); 32 sources of 1024^2 11.0 ms at 2, 11.2 at 4, 11.6 at 16; 3D 1.80 ms (97 x 131 x 203) and 8.6 ms
 // (checkerboard) at 0.4, 1.74 and 9.0 at 0.75, 1.75 and 9.7 at 1.5.
