@@ -39,6 +39,7 @@
 #include "eik_grid.cuh"
 #include "eik_internal.h"
 #define EIK_SCHED_FN __device__ __noinline__
+#define EIK_SCHED_PROGRESS 1
 #include "eik_sched.cuh"
 
 namespace eik {

@@ -94,8 +94,7 @@ struct SolveParams {
                                   // them, 2: and leave activations to a warp of their own
   Ctl *ctl;
   long long timeout_ns;
-  const unsigned long long *progress;   // a count that grows while work is done anywhere (NULL: a
-                                  // CTA's own wait alone counts against timeout_ns)
+  const unsigned long long *progress;   // adjoint: a count that grows while work is done anywhere
   int counters;
   int test_stall;
   unsigned window;                // buckets above the lowest active one that may be popped
