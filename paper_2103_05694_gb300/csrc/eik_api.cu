@@ -1315,8 +1315,8 @@ eik_status eik_sum_ordered(const double *const *src, int k, double *dst, int64_t
 // are solved (501 x 1201 cells in 4 slabs, 8 epochs: 49 -> 17 ms).  Ghost values
 // only decrease from epoch to epoch (the solve is monotone in its boundary
 // values), so the loop ends; a ghost whose neighbour has no value yet is an
-// ordinary cell, and one whose slab found a smaller value keeps that (its owner
-// then finds the same or less).  The fields never lie above those of epochs that
+// ordinary cell unless it is a source, and one whose slab found a smaller value keeps
+// that (its owner then finds the same or less).  The fields never lie above those of epochs that
 // start from +inf, so there are no more epochs than with these.  At the
 // end every cell of every slab satisfies the update with its neighbours'
 // final values across the slab boundaries, i.e. the union is the fixed point
@@ -1359,6 +1359,15 @@ eik_status eik_solve_slabs(const double *speed, double h, int ndim, const int64_
   CK(ws().slab_t.ensure((size_t)std::max<int64_t>(tcells, 1)), "slabs: fields");
   CK(ws().slab_x.ensure((size_t)std::max<int64_t>(nx_rows * plane, 1)), "slabs: exchange");
   std::vector<double> xprev((size_t)(nx_rows * plane), INFINITY), xcur((size_t)(nx_rows * plane));
+  // A source in a boundary row is fixed in both slabs from the first epoch on: as an
+  // ordinary ghost it could fall below its time, and would keep that value.
+  for (size_t i = 0; i < hp.src.size(); ++i) {
+    const int64_t row = hp.src[i] / plane, j = hp.src[i] % plane;
+    for (int b = 0; b + 1 < K; ++b) {
+      if (row == lo[b + 1] - 1) xprev[(size_t)(2 * b * plane + j)] = hp.t0[i];
+      if (row == lo[b + 1]) xprev[(size_t)((2 * b + 1) * plane + j)] = hp.t0[i];
+    }
+  }
   const int max_epochs = 64 + 8 * K;
   eik_stats acc;
   std::memset(&acc, 0, sizeof(acc));
