@@ -42,6 +42,15 @@
 namespace eik {
 namespace {
 
+// The time (bits) below which a visit accepts candidates while `lo` is the lowest
+// active bucket: the end of the look-ahead window.  The last bucket holds every
+// later time, so there is no limit where the window reaches it: the candidates
+// beyond one would be deferred to that bucket for ever.
+__device__ __forceinline__ unsigned long long visit_limit(unsigned lo, unsigned window, double delta) {
+  if (lo >= kMaxBucket || window >= kMaxBucket - lo) return kInfBits;
+  return bits_of(static_cast<double>(lo + window + 1u) * delta);
+}
+
 // ---------------------------------------------------------------------------
 // Persistent kernel: pop a tile, relax it in shared memory, commit, activate
 // neighbour tiles, repeat until no work is left anywhere.
@@ -168,8 +177,7 @@ __global__ void __launch_bounds__(TX * TY * TZ, WIDE ? EIK_WIDE_CTAS_64 : reside
           prob = find_prob(p, static_cast<unsigned long long>(tile));
           if (visit_budget && atomicAdd(&p.ctl->visits_total, 1ull) >= visit_budget)
             raise_status(p.ctl, kEtimeout, 9);   // this visit runs; then every CTA stops
-          const double vlim = static_cast<double>(lo + p.window + 1u) * s_delta;
-          s_vlim = bits_of(vlim);
+          s_vlim = visit_limit(lo, p.window, s_delta);
           const Prob &P = p.probs[prob];
           const long long lt = tile - P.tile_base;
           const long long rest = lt / P.ntx;
@@ -558,7 +566,7 @@ __global__ void __launch_bounds__(TX * TY * TZ, WIDE ? EIK_WIDE_CTAS_64 : reside
       }
       if (!cont && m < kInfBits) {
         const unsigned lo2 = ld_rlx(&p.ctl->cur);
-        const unsigned long long v2 = bits_of(static_cast<double>(lo2 + p.window + 1u) * s_delta);
+        const unsigned long long v2 = visit_limit(lo2, p.window, s_delta);
         if (m < v2) {
           cont = 2;
           s_faces = 0;

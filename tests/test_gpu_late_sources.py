@@ -86,3 +86,17 @@ def test_noalloc(shape):
         visits.append(stats["visits"])
     assert np.array_equal(_bits(out.cpu().numpy()), _bits(oracle.fmm(speed, 0.5, src, times).t))
     assert visits[1] < 2 * visits[0]
+
+
+@pytest.mark.parametrize("opts", [None, {"arith": 1}, {"arith": 2}, {"counters": 1}, {"arith": 1, "window": 1}])
+@pytest.mark.parametrize("shape", [(5, 6), (90, 110), (4, 4, 4), (20, 22, 25)])
+def test_beyond_the_last_bucket(shape, opts):
+    """Times of more than 2^30 bucket widths share the last bucket."""
+    rng = np.random.Generator(np.random.PCG64(4))
+    speed = rng.uniform(1.0, 4.0, shape)
+    src = np.sort(rng.choice(speed.size, 9, replace=False)).astype(np.int64)
+    times = 1e12 + rng.random(9)
+    want = oracle.fmm(speed, 0.5, src, times).t
+    r = eik.solve(torch.from_numpy(speed).to(DEV), 0.5, src, torch.from_numpy(times).to(DEV),
+                  opts=dict(opts or {}, timeout_ms=5000))
+    assert np.array_equal(_bits(r.t.cpu().numpy()), _bits(want))
