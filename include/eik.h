@@ -323,7 +323,8 @@ eik_status eik_adjoint(const eik_problem *probs, int nprob, const double *const 
  * ghost row on each side it shares with a neighbour, is one problem of a batch
  * (one persistent launch for all slabs).  A ghost row holds the neighbour's
  * values of those cells from the previous epoch as fixed sources (cells the
- * neighbour has not reached yet stay free).  Between epochs the rows next to
+ * neighbour has not reached yet stay free, but for its sources, which are fixed at
+ * their times from the first epoch on).  Between epochs the rows next to
  * each slab boundary are copied, device to device, into an exchange buffer;
  * the epochs repeat until no exchanged value changes (a global AND over the
  * boundaries).  Ghost values only decrease from epoch to epoch, so the loop
